@@ -26,6 +26,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "claire_internal.cuh"
@@ -267,23 +268,26 @@ __device__ __forceinline__ float gather_lean(const T *__restrict__ f, const Dims
 
 // ---------------------------------------------------------------------------
 // Software-pipelined tiled semi-Lagrangian step (the production path).
-// Persistent blocks walk the tiles of 32 x 8 x 4 voxels.  Every tile has a box
-// entry (written by the foot-point kernel with the displacements, or by
-// k_tile_ranges): the smallest floor of its displacements per axis, which
+// Blocks walk consecutive tiles of 32 x 8 x 4 voxels (sl_chunk).  Every tile
+// has a box entry (written by the foot-point kernel with the displacements, or
+// by k_tile_ranges): the smallest floor of its displacements per axis, which
 // fixes where its shared-memory source box starts, and whether the floors
 // fit the box.  While a block computes tile k from one shared-memory buffer,
-// cp.async already copies the box of tile k+1 into the other.  The
-// displacements and epilogue inputs of a tile are loaded when the tile starts,
-// not a tile ahead: that holds half the registers (three blocks per SM for the
-// incremental state, which has six epilogue inputs a voxel), and the loads
-// still overlap the box wait and the other resident blocks (measured at
-// 256^3: state 199 -> 182 us, adjoint 205 -> 187 us, incremental state
-// 234 -> 207 us, accumulating adjoint 242 -> 230 us).  The 64 taps of
-// a voxel are then shared-memory reads with immediate offsets, the same
-// instruction stream for every lane (the periodic wrap happened once, when
-// the box was fetched).  A tile whose floors span more than the box gathers
-// from global memory instead (the decision is uniform per tile), so a region
-// of large displacements slows only its own tiles.
+// cp.async already copies the box of tile k+1 into the other; one barrier per
+// tile orders both.  The displacements and epilogue inputs of a tile are
+// loaded when the tile starts: registers refilled voxel by voxel for the next
+// tile measured slower (state 194 -> 221 us, accumulating adjoint 250 -> 304:
+// the pending loads hold up the shared loads behind them).  The 64 taps of a
+// voxel are shared-memory reads with immediate offsets, the same instruction
+// stream for every lane (the periodic wrap happened once, when the box was
+// fetched).  A thread sums two voxels at a time on the paired FP32
+// instructions, weights included (212 warp instructions per 32 voxels instead
+// of 266).  What bounds the state step is the shared-memory pipe: 64 tap
+// wavefronts per 32 voxels, 10 more of bank conflicts where floors change
+// inside a warp and 8 of box copies and global accesses take 140 us at 256^3;
+// it runs in 181.  A tile whose floors span more than the box gathers from
+// global memory instead (the decision is uniform per tile), so a region of
+// large displacements slows only its own tiles.
 // ---------------------------------------------------------------------------
 constexpr int PT3 = 32, PT2 = 8, PT1 = 4;
 // box geometry, fixed at compile time: floors of a tile's displacements may
@@ -396,7 +400,10 @@ __device__ __forceinline__ void sl_load_epi(const A &a, long long id, long long 
 }
 
 // Box copy of tile rows [lo1, lo1 + BS1) x [lo2, lo2 + BS2) x [lo3, lo3 + BS3)
-// of a periodic field.  Chunked (n3 a multiple of 4 and a 16-byte aligned
+// of a periodic field (the caller commits the copies).  A box whose rows do not
+// wrap along x1 and x2 steps from row to row with one add (foot points 858 ->
+// 740 us per call at 256^3, both sides; the wrapping rows' divisions were a
+// tenth of the SL steps' instructions).  Chunked (n3 a multiple of 4 and a 16-byte aligned
 // field): 16-byte cp.async of 40 floats per row from lo3 rounded down to a
 // multiple of 4, three rows per warp instruction; the stencil columns then sit
 // box_shift() floats further right.  Otherwise one float per lane and column.
@@ -420,13 +427,39 @@ __device__ __forceinline__ void box_copy(const float *__restrict__ src, const Di
         const int lrow = tx / BOX_CH, lch = tx - lrow * BOX_CH;
         if (tx < 3 * BOX_CH) {
             const int gx = wrap_index((lo3 & ~3) + 4 * lch, d.n3);
+            constexpr int STEP = 3 * PT2, IT = (BOX_ROWS + STEP - 1) / STEP;  // rows per sweep of the block, sweeps
+            const int row0 = 3 * ty + lrow;
+            int z = row0 / BS2, y = row0 - z * BS2;
+            float *dst = buf + row0 * BOX_PITCH + 4 * lch;
+            if (lo1 >= 0 && lo2 >= 0 && lo1 + BS1 <= d.n1 && lo2 + BS2 <= d.n2) {
+                // no row wraps: STEP rows further are one plane and STEP - BS2
+                // rows, or two planes and STEP - 2 BS2 rows (an offset fits an
+                // int: at most 1024^3 elements)
+                constexpr int DY = STEP - BS2;
+                static_assert(DY >= 0 && DY < BS2, "a sweep advances between one and two box planes");
+                int o = (lo1 + z) * (int)plane + (lo2 + y) * d.n3 + gx;
+                const int stepa = (int)plane + DY * d.n3, stepb = stepa + (int)plane - BS2 * d.n3;
 #pragma unroll
-            for (int i = 0; i < (BOX_ROWS + 3 * PT2 - 1) / (3 * PT2); ++i) {
-                const int row = 3 * (ty + PT2 * i) + lrow;
-                if (row < BOX_ROWS) {
-                    const int z = row / BS2, y = row - z * BS2;
-                    cp_async16(buf + row * BOX_PITCH + 4 * lch,
-                               src + wrap_index(lo1 + z, d.n1) * plane + (long long)wrap_index(lo2 + y, d.n2) * d.n3 + gx);
+                for (int i = 0; i < IT; ++i) {
+                    if (STEP * (i + 1) <= BOX_ROWS || row0 < BOX_ROWS - STEP * i)
+                        cp_async16(dst + i * STEP * BOX_PITCH, src + o);
+                    const bool two = y + DY >= BS2;
+                    o += two ? stepb : stepa;
+                    y += two ? DY - BS2 : DY;
+                }
+            } else {
+#pragma unroll 1
+                for (int i = 0; i < IT; ++i) {
+                    if (row0 < BOX_ROWS - STEP * i)
+                        cp_async16(dst, src + wrap_index(lo1 + z, d.n1) * plane +
+                                            (long long)wrap_index(lo2 + y, d.n2) * d.n3 + gx);
+                    dst += STEP * BOX_PITCH;
+                    y += STEP - BS2;
+                    ++z;
+                    if (y >= BS2) {
+                        y -= BS2;
+                        ++z;
+                    }
                 }
             }
         }
@@ -449,7 +482,6 @@ __device__ __forceinline__ void box_copy(const float *__restrict__ src, const Di
             }
         }
     }
-    cp_async_commit();
 }
 
 // 64-tap tricubic sum from a box position; pairs of rows go through the
@@ -477,6 +509,48 @@ __device__ __forceinline__ float box_cubic(const float *p, const float w1[4], co
     }
     return u.x + u.y;
 }
+
+// cubic Lagrange weights of two voxels at once (packed FP32 instructions)
+__device__ __forceinline__ void lagrange4x2(float2 t, float2 w[4]) {
+    const float2 tp1 = __fadd2_rn(t, make_float2(1.f, 1.f)), tm1 = __fadd2_rn(t, make_float2(-1.f, -1.f));
+    const float2 tm2 = __fadd2_rn(t, make_float2(-2.f, -2.f));
+    const float2 a = __fmul2_rn(t, tm2), b = __fmul2_rn(tp1, tm1);
+    const float s = 1.f / 6.f;
+    w[0] = __fmul2_rn(__fmul2_rn(make_float2(-s, -s), a), tm1);
+    w[1] = __fmul2_rn(__fmul2_rn(make_float2(0.5f, 0.5f), b), tm2);
+    w[2] = __fmul2_rn(__fmul2_rn(make_float2(-0.5f, -0.5f), tp1), a);
+    w[3] = __fmul2_rn(__fmul2_rn(make_float2(s, s), b), t);
+}
+
+// the tricubic sums of two voxels, voxel x at box position p, voxel y at q;
+// per voxel the same operations in the same order as box_cubic
+__device__ __forceinline__ float2 box_cubic2(const float *p, const float *q, const float2 w1[4], const float2 w2[4],
+                                             const float2 w3[4]) {
+    float2 ux = make_float2(0.f, 0.f), uy = ux;
+#pragma unroll
+    for (int ia = 0; ia < 4; ++ia) {
+        float2 s[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int o = (ia * BS2 + j) * BOX_PITCH;
+            float2 t = __fmul2_rn(w3[0], make_float2(p[o], q[o]));
+            t = __ffma2_rn(w3[1], make_float2(p[o + 1], q[o + 1]), t);
+            t = __ffma2_rn(w3[2], make_float2(p[o + 2], q[o + 2]), t);
+            s[j] = __ffma2_rn(w3[3], make_float2(p[o + 3], q[o + 3]), t);
+        }
+        const float2 tx = __ffma2_rn(s[2], w2[2], __fmul2_rn(s[0], w2[0]));
+        const float2 ty = __ffma2_rn(s[3], w2[3], __fmul2_rn(s[1], w2[1]));
+        ux = ia == 0 ? __fmul2_rn(tx, w1[0]) : __ffma2_rn(tx, w1[ia], ux);
+        uy = ia == 0 ? __fmul2_rn(ty, w1[0]) : __ffma2_rn(ty, w1[ia], uy);
+    }
+    return __fadd2_rn(ux, uy);
+}
+
+// floor of a displacement whose magnitude is below 2^22 without conversion
+// instructions: adding 1.5 * 2^23 rounded down leaves the floor in the low
+// mantissa bits.  bits(m) = FLOOR_BITS + floor, m - FLOOR_MAGIC = floor.
+constexpr float FLOOR_MAGIC = 12582912.f;
+constexpr unsigned FLOOR_BITS = 0x4B400000u;
 
 // trilinear sum from the cubic stencil origin p (nodes floor and floor + 1)
 __device__ __forceinline__ float box_linear(const float *p, float u1, float u2, float u3) {
@@ -587,7 +661,7 @@ constexpr int GTAB = 64;  // box entries a block stages in shared memory at a ti
 // tile needs a bounds check (measured ~5% of the step time at 256^3)
 template <int MODE, int ORDER, typename TS = float, typename TG = float, bool FULL = false>
 __global__ void __launch_bounds__(PT3 * PT2, SlOcc<MODE>::v)
-k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked_in) {
+k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked_in, int chunk) {
     static_assert(std::is_same<TS, float>::value, "the box path stages FP32 source fields");
     constexpr int NE = EpiCount<MODE>::v > 0 ? EpiCount<MODE>::v : 1;
     constexpr int NX = EarlyCount<MODE>::v > 0 ? EarlyCount<MODE>::v : 1;
@@ -598,45 +672,29 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
     const int nb3 = (d.n3 + PT3 - 1) / PT3, nb2 = (d.n2 + PT2 - 1) / PT2, nb1 = (d.n1 + PT1 - 1) / PT1;
     const int ntiles = nb3 * nb2 * nb1;
     const long long N = d.N, plane = (long long)d.n2 * d.n3;
-    int tbeg, tend;
-    tile_range(ntiles, tbeg, tend);
+    const int tbeg = min(ntiles, (int)blockIdx.x * chunk), tend = min(ntiles, tbeg + chunk);
     if (tbeg < tend) {
         // box of a tile at its own floor range g (lo1, lo2, lo3); a tile whose
-        // range does not fit (g.w == 0) copies nothing, but still commits a
-        // (empty) group so that the wait counts stay the same
+        // range does not fit (g.w == 0) copies nothing
         auto issue_box = [&](int t1, int t2, int t3, const int4 &g, float *buf) {
             if (g.w) box_copy(a.src, d, plane, t1 * PT1 + g.x - 1, t2 * PT2 + g.y - 1, t3 * PT3 + g.z - 1, buf, chunked);
-            else cp_async_commit();
         };
-        // displacements and epilogue inputs of the voxels of a tile
-        auto load_regs = [&](int t1, int t2, int t3, float *dd, float *ee) {
-            const int i3 = t3 * PT3 + tx, i2 = t2 * PT2 + ty;
-            const long long id0 = (long long)t1 * PT1 * plane + (long long)i2 * d.n3 + i3;
-#pragma unroll
-            for (int t = 0; t < PT1; ++t) {
-                if (FULL || (i3 < d.n3 && i2 < d.n2 && t1 * PT1 + t < d.n1)) {
-                    const long long id = id0 + t * plane;
-                    dd[3 * t] = a.disp[id];
-                    dd[3 * t + 1] = a.disp[N + id];
-                    dd[3 * t + 2] = a.disp[2 * N + id];
-                    sl_load_epi<MODE>(a, id, N, ee + NE * t);
-                }
-            }
-        };
-
-        // the block's box entries are staged in shared memory, GTAB at a time
-        // (a register copy of a pending global load would stall each tile)
-        __shared__ int4 gtab[GTAB];
+        // the block's box entries are staged in shared memory, two tables of
+        // GTAB in turn (a register copy of a pending global load would stall
+        // each tile)
+        __shared__ int4 gtab[2][GTAB];
         auto stage_entries = [&](int first) {
-            for (int k = ty * PT3 + tx; k < GTAB && first + k < tend; k += PT3 * PT2) gtab[k] = tiles[first + k];
+            const int k = ty * PT3 + tx;
+            if (k < GTAB && first + k < tend) gtab[((first - tbeg) / GTAB) & 1][k] = tiles[first + k];
         };
-        int gbase = tbeg;
-        stage_entries(gbase);
-        __syncthreads();
-        // tile counters of the next tile to fetch (x3 fastest)
+        auto entry = [&](int tile) { return gtab[((tile - tbeg) / GTAB) & 1][(tile - tbeg) % GTAB]; };
+        stage_entries(tbeg);
+        // coordinates of the current tile (x3 fastest)
         int c3 = tbeg % nb3, c2 = (tbeg / nb3) % nb2, c1 = tbeg / (nb3 * nb2);
-        int4 g_cur = gtab[0];
+        __syncthreads();
+        int4 g_cur = entry(tbeg);
         issue_box(c1, c2, c3, g_cur, smem);
+        cp_async_commit();
         int cur = 0;
         for (int tile = tbeg; tile < tend; ++tile) {
             const int t1 = c1, t2 = c2, t3 = c3;
@@ -644,74 +702,98 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
                 c3 = 0;
                 if (++c2 == nb2) { c2 = 0; ++c1; }
             }
-            // this tile's inputs, loaded now: they arrive while the box of
-            // the next tile is issued and this tile's box is awaited
-            float cd[PT1 * 3], ce[PT1 * NE], cx[PT1][NX];
-            load_regs(t1, t2, t3, cd, ce);
             const int i3 = t3 * PT3 + tx, i2 = t2 * PT2 + ty;
             const long long id0 = (long long)t1 * PT1 * plane + (long long)i2 * d.n3 + i3;
             const bool inplane = FULL || (i3 < d.n3 && i2 < d.n2);
-            if (EarlyCount<MODE>::v > 0 && inplane) {
+            // the tile's displacements and epilogue inputs, loaded now: they
+            // arrive while its box is awaited and the next one is issued
+            float cd[PT1][3], ce[PT1][NE], cx[PT1][NX];
 #pragma unroll
-                for (int t = 0; t < PT1; ++t)
-                    if (FULL || t1 * PT1 + t < d.n1) sl_load_early<MODE>(a, id0 + t * plane, N, cx[t]);
-            }
-            // entry of the next tile (the table is refilled behind the barrier
-            // that follows this tile when the next tile starts a new batch)
-            const int4 g_next = tile + 1 < tend && tile + 1 - gbase < GTAB ? gtab[tile + 1 - gbase] : g_cur;
-            const bool refill = tile + 1 < tend && tile + 1 - gbase == GTAB;
-            if (tile + 1 < tend) {
-                if (refill) {
-                    // the next batch of entries: its first one is read here
-                    // from global memory, the rest after the end barrier
-                    const int4 gn = tiles[tile + 1];
-                    issue_box(c1, c2, c3, gn, smem + (cur ^ 1) * BOX_FLOATS);
+            for (int t = 0; t < PT1; ++t) {
+                if (FULL || (inplane && t1 * PT1 + t < d.n1)) {
+                    const long long id = id0 + t * plane;
+                    cd[t][0] = a.disp[id];
+                    cd[t][1] = a.disp[N + id];
+                    cd[t][2] = a.disp[2 * N + id];
+                    sl_load_epi<MODE>(a, id, N, ce[t]);
+                    sl_load_early<MODE>(a, id, N, cx[t]);
                 } else {
-                    issue_box(c1, c2, c3, g_next, smem + (cur ^ 1) * BOX_FLOATS);
+                    // a voxel outside the grid: any position inside the box
+                    cd[t][0] = g_cur.x;
+                    cd[t][1] = g_cur.y;
+                    cd[t][2] = g_cur.z;
                 }
-                cp_async_wait<1>();
-            } else {
-                cp_async_wait<0>();
             }
+            // One barrier per tile: behind it every thread's part of this
+            // tile's box has arrived and every thread has finished the tile
+            // before, so the other buffer (and the other entry table) is free.
+            cp_async_wait<0>();
             __syncthreads();
-            const float *bx = smem + cur * BOX_FLOATS;
-            const int fmn0 = g_cur.x, fmn1 = g_cur.y, fmn2 = g_cur.z;
-            const int sh = box_shift(t3 * PT3 + fmn2 - 1, chunked);
+            if ((tile - tbeg) % GTAB == 0) stage_entries(tile + GTAB);
+            int4 g_next = g_cur;
+            if (tile + 1 < tend) {
+                g_next = entry(tile + 1);
+                issue_box(c1, c2, c3, g_next, smem + (cur ^ 1) * BOX_FLOATS);
+                cp_async_commit();
+            }
             if (!g_cur.w) {
                 const Acc2 td = sl_gather_tile<MODE, ORDER>(a, d, t1, t2, t3);
                 if (MODE == SL_ADJDOT) dot.add(td.s, td.c);
             } else if (inplane) {
+                // box position of this thread's voxel 0 at floors 0, less the
+                // constant part of the floor bits (unsigned: wraps)
+                const int sh = box_shift(t3 * PT3 + g_cur.z - 1, chunked);
+                const unsigned e0 = (unsigned)(cur * BOX_FLOATS + (ty - g_cur.x * BS2 - g_cur.y) * BOX_PITCH + tx -
+                                               g_cur.z + sh) -
+                                    FLOOR_BITS * (unsigned)(BS2 * BOX_PITCH + BOX_PITCH + 1);
 #pragma unroll
-                for (int t = 0; t < PT1; ++t) {
-                    if (FULL || t1 * PT1 + t < d.n1) {
-                        const float *dt3 = cd + 3 * t;
-                        const float fl0 = floorf(dt3[0]), fl1 = floorf(dt3[1]), fl2 = floorf(dt3[2]);
-                        // stencil origin inside the box; every tap is an immediate offset
-                        const int b1 = t + (int)fl0 - fmn0, b2 = ty + (int)fl1 - fmn1, b3 = tx + (int)fl2 - fmn2 + sh;
-                        const float *p = bx + (b1 * BS2 + b2) * BOX_PITCH + b3;
-                        float acc = 0.f;
-                        if (!box_origin_ok(b1, b2, b3, box_cols(chunked))) {
-                        } else if (ORDER == 1) {
-                            acc = box_linear(p, dt3[0] - fl0, dt3[1] - fl1, dt3[2] - fl2);
+                for (int t = 0; t < PT1; t += 2) {
+                    const bool ok0 = FULL || t1 * PT1 + t < d.n1, ok1 = FULL || t1 * PT1 + t + 1 < d.n1;
+                    const long long id = id0 + t * plane;
+                    float2 u[3];
+                    unsigned o[2];
+                    bool in[2];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const float *dd = cd[t + k];
+                        const float m0 = __fadd_rd(dd[0], FLOOR_MAGIC), m1 = __fadd_rd(dd[1], FLOOR_MAGIC);
+                        const float m2 = __fadd_rd(dd[2], FLOOR_MAGIC);
+                        const float r0 = dd[0] - (m0 - FLOOR_MAGIC), r1 = dd[1] - (m1 - FLOOR_MAGIC);
+                        const float r2 = dd[2] - (m2 - FLOOR_MAGIC);
+                        if (k == 0) {
+                            u[0].x = r0;
+                            u[1].x = r1;
+                            u[2].x = r2;
                         } else {
-                            float w1[4], w2[4], w3[4];
-                            lagrange4(dt3[0] - fl0, w1);
-                            lagrange4(dt3[1] - fl1, w2);
-                            lagrange4(dt3[2] - fl2, w3);
-                            acc = box_cubic(p, w1, w2, w3);
+                            u[0].y = r0;
+                            u[1].y = r1;
+                            u[2].y = r2;
                         }
-                        sl_epilogue<MODE>(a, id0 + t * plane, N, acc, ce + NE * t, cx[t], dot);
+                        const unsigned f0 = __float_as_uint(m0), f1 = __float_as_uint(m1), f2 = __float_as_uint(m2);
+                        o[k] = e0 + (unsigned)((t + k) * BS2 * BOX_PITCH) + f0 * (unsigned)(BS2 * BOX_PITCH) +
+                               f1 * (unsigned)BOX_PITCH + f2;
+                        in[k] = box_origin_ok(t + k + (int)(f0 - FLOOR_BITS) - g_cur.x,
+                                              ty + (int)(f1 - FLOOR_BITS) - g_cur.y,
+                                              tx + (int)(f2 - FLOOR_BITS) - g_cur.z + sh, box_cols(chunked));
                     }
+                    float2 acc = make_float2(0.f, 0.f);
+                    if (!(in[0] && in[1])) {
+                    } else if (ORDER == 1) {
+                        acc.x = box_linear(smem + o[0], u[0].x, u[1].x, u[2].x);
+                        acc.y = box_linear(smem + o[1], u[0].y, u[1].y, u[2].y);
+                    } else {
+                        float2 w1[4], w2[4], w3[4];
+                        lagrange4x2(u[0], w1);
+                        lagrange4x2(u[1], w2);
+                        lagrange4x2(u[2], w3);
+                        acc = box_cubic2(smem + o[0], smem + o[1], w1, w2, w3);
+                    }
+                    if (ok0) sl_epilogue<MODE>(a, id, N, acc.x, ce[t], cx[t], dot);
+                    if (ok1) sl_epilogue<MODE>(a, id + plane, N, acc.y, ce[t + 1], cx[t + 1], dot);
                 }
             }
-            __syncthreads();
+            g_cur = g_next;
             cur ^= 1;
-            if (refill) {
-                gbase = tile + 1;
-                stage_entries(gbase);
-                __syncthreads();
-            }
-            g_cur = gtab[tile + 1 - gbase < GTAB ? tile + 1 - gbase : 0];
         }
     }
     sl_dot_store<MODE>(dot, a.partial);
@@ -839,10 +921,11 @@ k_footpoints_box(const float *__restrict__ v, float *__restrict__ dispm, float *
             const bool fits = rng[1] - f0 <= BOX_SPAN && rng[3] - f1 <= BOX_SPAN && rng[5] - f2 <= BOX_SPAN &&
                               floor_sane(f0, rng[1]) && floor_sane(f1, rng[3]) && floor_sane(f2, rng[5]);
             if (fits) {
-#pragma unroll
+#pragma unroll 1
                 for (int c = 0; c < 3; ++c)
                     box_copy(v + c * N, d, plane, t1 * PT1 + f0 - 1, t2 * PT2 + f1 - 1, t3 * PT3 + f2 - 1,
                              smem + c * BOX_FLOATS, chunked);
+                cp_async_commit();
                 cp_async_wait<0>();
                 __syncthreads();
             }
@@ -922,6 +1005,24 @@ inline int pipe_blocks(const Dims &d, int per_sm) {
     return (int)(ntiles < want ? ntiles : want);
 }
 
+// Consecutive tiles per block of an SL step with `slots` resident blocks on
+// the chip.  Tiles take different times (crossing floors conflict in shared
+// memory, dies differ in distance to memory), so on large grids blocks of a few
+// tiles handed out by the hardware as others finish beat one equal share per
+// resident block, whose SMs ran at 79% of their warps towards the end: state
+// 190 -> 181 us at 256^3 and 92 -> 86 at 192^3 with 4 tiles a block (8: 184,
+// 88); the accumulating adjoint steps (two blocks per SM) 240 -> 234 at 256^3
+// with 8 (4: 236), and no gain at 192^3 (109 both).  A new block exposes its
+// first loads, so with fewer tiles to a slot (128^3: 4.5; state 33.7 with equal
+// shares, 35.5 with 4 tiles) every block takes an equal share of one wave.
+// At most 4 kReduceBlocks blocks: a dot-product step leaves one partial sum each.
+inline int sl_chunk(long long ntiles, int slots, bool two_per_sm) {
+    const int few = two_per_sm ? 8 : 4;
+    const long long share = (ntiles + slots - 1) / slots;
+    const long long chunk = share > (two_per_sm ? 32 : 12) ? few : share;
+    return (int)std::max<long long>(chunk, (ntiles + 4 * kReduceBlocks - 1) / (4 * kReduceBlocks));
+}
+
 // returns the number of blocks launched (the partial sums a dot-product step
 // leaves for its finalize)
 template <int MODE, int ORDER, typename TS, typename TG, bool FULL>
@@ -930,8 +1031,9 @@ int launch_pipe_f(const Dims &d, const SlArgsT<TS, TG> &a, const int4 *tiles, cu
     // the shared-memory limit is set once per instantiation and device
     static SmemAttr attr;
     attr.ensure(k_sl_pipe<MODE, ORDER, TS, TG, FULL>, (int)smem, "k_sl_pipe");
-    const int grid = pipe_blocks(d, SlOcc<MODE>::v);
-    k_sl_pipe<MODE, ORDER, TS, TG, FULL><<<grid, dim3(PT3, PT2), smem, st>>>(a, d, tiles, chunk_ok(d, a.src));
+    const int chunk = sl_chunk(tile_count(d), SlOcc<MODE>::v * num_sms(), SlOcc<MODE>::v == 2);
+    const int grid = (int)((tile_count(d) + chunk - 1) / chunk);
+    k_sl_pipe<MODE, ORDER, TS, TG, FULL><<<grid, dim3(PT3, PT2), smem, st>>>(a, d, tiles, chunk_ok(d, a.src), chunk);
     return grid;
 }
 
