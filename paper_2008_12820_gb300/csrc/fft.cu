@@ -25,7 +25,7 @@
 #include <type_traits>
 
 #include "claire_internal.cuh"
-#include "fft_core.cuh"
+#include "fft_reg.cuh"
 
 namespace claire {
 
@@ -242,8 +242,9 @@ __device__ __forceinline__ void mul_point(float2 &pa, float2 &pb, float2 &pc, fl
         const float2 a = pa, b = pb, c = pc;
         const float kk = k1 * k1 + k2 * k2 + k3 * k3;
         const float kd2 = k1d * k1d + k2d * k2d + k3d * k3d;
-        const float2 kv = make_float2(k1d * a.x + k2d * b.x + k3d * c.x,
-                                      k1d * a.y + k2d * b.y + k3d * c.y);
+        // fused products spelled out: every pass rounds alike
+        const float2 kv = make_float2(__fmaf_rn(k3d, c.x, __fmaf_rn(k1d, a.x, __fmul_rn(k2d, b.x))),
+                                      __fmaf_rn(k3d, c.y, __fmaf_rn(k1d, a.y, __fmul_rn(k2d, b.y))));
         float diag, coup;
         if (OP == OP_A) {
             diag = sp.beta * kk;
@@ -259,9 +260,14 @@ __device__ __forceinline__ void mul_point(float2 &pa, float2 &pb, float2 &pc, fl
             }
         }
         const float s = sp.scale;
-        pa = make_float2((diag * a.x + coup * k1d * kv.x) * s, (diag * a.y + coup * k1d * kv.y) * s);
-        pb = make_float2((diag * b.x + coup * k2d * kv.x) * s, (diag * b.y + coup * k2d * kv.y) * s);
-        pc = make_float2((diag * c.x + coup * k3d * kv.x) * s, (diag * c.y + coup * k3d * kv.y) * s);
+        auto row = [&](float kd, const float2 &v) {
+            const float ck = __fmul_rn(coup, kd);
+            return make_float2(__fmul_rn(__fmaf_rn(diag, v.x, __fmul_rn(ck, kv.x)), s),
+                               __fmul_rn(__fmaf_rn(diag, v.y, __fmul_rn(ck, kv.y)), s));
+        };
+        pa = row(k1d, a);
+        pb = row(k2d, b);
+        pc = row(k3d, c);
     }
 }
 
@@ -544,6 +550,293 @@ k_c2r_x3_p(const float2 *__restrict__ in, TO *__restrict__ out, const float *__r
     }
 }
 
+// ------------------------------------------- register-resident passes ----
+// The same five passes for the lengths N = 16 G (fft_reg.cuh): one tile per
+// block, read from and written to global memory by the register steps
+// themselves, so a pass has one exchange through shared memory per transform
+// (x1 with the multiplier: two for both transforms where G divides 16) and
+// three blocks per SM hide one another's loads.  The staged, double-buffered
+// forms they replace at these lengths were bound by shared-memory round trips,
+// barriers and issue.  Per pass over three components, before and after:
+//   256^3 (59 us at the copy rate)  x3 forward 90 -> 66 us, x2 81 -> 70,
+//         x1 with multiplier 145 -> 121, x3 inverse 117 -> 78 (with addend)
+//   192^3 (25 us)  50 -> 36, 61 -> 32, 93 -> 54, 64 -> 40
+//   128^3 (7.5 us, and about 5 us of launch)  19 -> 15, 16.5 -> 12, 26 -> 19, 21 -> 13
+// The x3 and x2 passes are within 0.75-0.9 of the copy rate at 256^3; the x1
+// pass is bound by its registers (96 data values a thread, 12 warps per SM).
+
+// x2 transform (S = 0: direction s) and the x1 transform without a multiplier
+// (S = -1 forward, S = +1 inverse of the elements times `scale`), in place
+template <int N, int S>
+__global__ void __launch_bounds__(RegTile<N>::T, 768 / RegTile<N>::T)
+kr_c2c(float2 *__restrict__ data, const float2 *__restrict__ tw, RegLines q, float s, float scale) {
+    using P = RegPlan<N>;
+    constexpr int TL = RegTile<N>::TL, T = RegTile<N>::T, G = P::G;
+    __shared__ float2 w[P::W];
+    __shared__ float2 sm[P::ROWS * TL];
+    reg_twiddles<N, T>(w, tw);
+    const int l = threadIdx.x % TL, j = threadIdx.x / TL;
+    long long off;
+    int col;
+    const bool ok = reg_line(q, blockIdx.x * TL + l, off, col);
+    float2 *base = data + off + col;
+    if (P::P2 || j < G) {
+        float2 a[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) a[r] = ok ? base[(j + G * r) * q.estride] : make_float2(0.f, 0.f);
+        if (S > 0) {
+#pragma unroll
+            for (int r = 0; r < 16; ++r) a[r] = make_float2(__fmul_rn(a[r].x, scale), __fmul_rn(a[r].y, scale));
+        }
+        dft<16>(a, S == 0 ? s : (float)S);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) sm[(17 * j + r) * TL + l] = a[r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 16 / P::TPL; ++i) {
+        const int k = j + P::TPL * i;
+        float2 a[G];
+#pragma unroll
+        for (int m = 0; m < G; ++m) a[m] = sm[(k + 17 * m) * TL + l];
+        reg_step2<N, S>(a, k, w, s);
+        if (ok) {
+#pragma unroll
+            for (int m = 0; m < G; ++m) base[(k + 16 * m) * q.estride] = a[m];
+        }
+    }
+}
+
+// x3 forward, two real lines as one complex line; Z_{n-k} of the Hermitian
+// split comes from the lane that holds it
+template <int N>
+__global__ void __launch_bounds__(RegTile<N>::T, 768 / RegTile<N>::T)
+kr_r2c(const float *__restrict__ in, float2 *__restrict__ out, const float2 *__restrict__ tw, long long nlines,
+       int p3) {
+    using P = RegPlan<N>;
+    constexpr int TL = RegTile<N>::TL, T = RegTile<N>::T, G = P::G;
+    __shared__ float2 w[P::W];
+    __shared__ float2 sm[P::ROWS * TL];
+    reg_twiddles<N, T>(w, tw);
+    if (threadIdx.x < G * TL) {
+        const int j = threadIdx.x % G, l = threadIdx.x / G;
+        const long long la = 2 * ((long long)blockIdx.x * TL + l);
+        const float *pa = in + la * N + j;
+        const bool ok0 = la < nlines, ok1 = la + 1 < nlines;
+        float2 a[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r)
+            a[r] = make_float2(ok0 ? __ldg(pa + G * r) : 0.f, ok1 ? __ldg(pa + N + G * r) : 0.f);
+        dft<16>(a, -1.f);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) sm[l * P::ROWS + 17 * j + r] = a[r];
+    }
+    __syncthreads();
+    const int k = threadIdx.x % 16;
+    const int src = ((threadIdx.x & 31) & 16) | ((16 - k) & 15);  // lane of index n - k
+#pragma unroll
+    for (int i = 0; i < 16 / P::TPL; ++i) {
+        const int l = threadIdx.x / 16 + i * (T / 16);
+        float2 a[G];
+#pragma unroll
+        for (int m = 0; m < G; ++m) a[m] = sm[l * P::ROWS + k + 17 * m];
+        reg_step2<N, -1>(a, k, w);
+        const long long la = 2 * ((long long)blockIdx.x * TL + l);
+        float2 *oa = out + la * p3 + k;
+        const bool ok0 = la < nlines, ok1 = la + 1 < nlines;
+#pragma unroll
+        for (int m = 0; m <= G / 2; ++m) {
+            // element k + 16 m (m = G / 2: only k = 0) and its mirror
+            const float2 z = a[m];
+            float2 zn;
+            zn.x = __shfl_sync(0xffffffffu, a[G - 1 - m].x, src);
+            zn.y = __shfl_sync(0xffffffffu, a[G - 1 - m].y, src);
+            if (k == 0) zn = a[(G - m) % G];
+            const float2 fa = make_float2(0.5f * (z.x + zn.x), 0.5f * (z.y - zn.y));
+            const float2 fb = make_float2(0.5f * (z.y + zn.y), -0.5f * (z.x - zn.x));
+            if (m < G / 2 || k == 0) {
+                if (ok0) oa[16 * m] = fa;
+                if (ok1) oa[p3 + 16 * m] = fb;
+            }
+        }
+    }
+}
+
+// x3 inverse; every stored coefficient k gives Z_k = A_k + i B_k and its mirror
+template <int N, int EPI>
+__global__ void __launch_bounds__(RegTile<N>::T, 768 / RegTile<N>::T)
+kr_c2r(const float2 *__restrict__ in, float *out, const float *add, const float2 *__restrict__ tw, long long nlines,
+       int p3) {
+    using P = RegPlan<N>;
+    constexpr int TL = RegTile<N>::TL, T = RegTile<N>::T, G = P::G;
+    __shared__ float2 w[P::W];
+    __shared__ float2 sm[P::ROWS * TL];
+    reg_twiddles<N, T>(w, tw);
+    if (threadIdx.x < G * TL) {
+        const int j = threadIdx.x % G, l = threadIdx.x / G;
+        const long long la = 2 * ((long long)blockIdx.x * TL + l);
+        const float2 *pa = in + la * p3;
+        const bool ok0 = la < nlines, ok1 = la + 1 < nlines;
+        const float2 zero = make_float2(0.f, 0.f);
+        float2 a[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const int e = j + G * r;
+            const bool lo = r < 8 || (r == 8 && j == 0);  // e <= N / 2
+            const int k = lo ? e : N - e;
+            float2 fa = ok0 ? __ldg(pa + k) : zero, fb = ok1 ? __ldg(pa + p3 + k) : zero;
+            if ((r == 0 || r == 8) && j == 0) {
+                fa.y = 0.f;
+                fb.y = 0.f;
+            }
+            a[r] = lo ? make_float2(fa.x - fb.y, fa.y + fb.x) : make_float2(fa.x + fb.y, -fa.y + fb.x);
+        }
+        dft<16>(a, 1.f);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) sm[l * P::ROWS + 17 * j + r] = a[r];
+    }
+    __syncthreads();
+    const int k = threadIdx.x % 16;
+#pragma unroll
+    for (int i = 0; i < 16 / P::TPL; ++i) {
+        const int l = threadIdx.x / 16 + i * (T / 16);
+        const long long la = 2 * ((long long)blockIdx.x * TL + l);
+        const bool ok0 = la < nlines, ok1 = la + 1 < nlines;
+        float2 a[G], g[G];
+#pragma unroll
+        for (int m = 0; m < G; ++m) a[m] = sm[l * P::ROWS + k + 17 * m];
+        if (EPI == EPI_ADD) {
+#pragma unroll
+            for (int m = 0; m < G; ++m)
+                g[m] = make_float2(ok0 ? add[la * N + k + 16 * m] : 0.f, ok1 ? add[(la + 1) * N + k + 16 * m] : 0.f);
+        }
+        reg_step2<N, 1>(a, k, w);
+#pragma unroll
+        for (int m = 0; m < G; ++m) {
+            if (ok0) out[la * N + k + 16 * m] = EPI == EPI_ADD ? a[m].x + g[m].x : a[m].x;
+            if (ok1) out[(la + 1) * N + k + 16 * m] = EPI == EPI_ADD ? a[m].y + g[m].y : a[m].y;
+        }
+    }
+}
+
+// x1 forward, multiplier, x1 inverse, in place.  A thread holds the same
+// elements of all three components, so the coupled multiplier needs no
+// exchange of its own.
+template <int N>
+struct RegMul {
+    static constexpr int TL = N == 32 ? 16 : 8;
+    static constexpr int T = RegPlan<N>::TPL * TL;
+    // resident threads per SM that the registers are cut for: 168 registers
+    // (384) at 256 and the composite lengths, 255 (256) where the smaller
+    // blocks spill more than the third block hides (x1 pass at 128^3 22.3 ->
+    // 19.2 us, at 256^3 121 against 124)
+    static constexpr int PER_SM = N == 256 || !RegPlan<N>::P2 ? 384 : 256;
+    static constexpr size_t smem = (size_t)(3 * RegPlan<N>::ROWS * TL + RegPlan<N>::W) * sizeof(float2);
+};
+template <int N, int OP>
+__global__ void __launch_bounds__(RegMul<N>::T, RegMul<N>::PER_SM / RegMul<N>::T)
+kr_mul(float2 *__restrict__ data, const float2 *__restrict__ tw, RegLines q, int n2, int n3, SpecParams sp) {
+    using P = RegPlan<N>;
+    constexpr int TL = RegMul<N>::TL, T = RegMul<N>::T, G = P::G, CS = P::ROWS * TL;
+    extern __shared__ float2 sm[];
+    float2 *w = sm + 3 * CS;
+    reg_twiddles<N, T>(w, tw);
+    const int l = threadIdx.x % TL, j = threadIdx.x / TL;
+    long long off;
+    int col;
+    const int line = blockIdx.x * TL + l, i2 = line / q.ncol;
+    const bool ok = reg_line(q, line, off, col);
+    float2 *base = data + off + col;
+    const bool act = P::P2 || j < G;
+    float2 a[3][16];
+    if (act) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int r = 0; r < 16; ++r)
+                a[c][r] = ok ? base[c * q.cstride + (j + G * r) * q.estride] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            dft<16>(a[c], -1.f);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) sm[c * CS + (17 * j + r) * TL + l] = a[c][r];
+        }
+    }
+    __syncthreads();
+    const float k2 = wavenumber(i2, n2), k2d = wavenumber_d1(i2, n2);
+    const float k3 = (float)col, k3d = ((n3 & 1) == 0 && 2 * col == n3) ? 0.f : k3;
+    auto mul = [&](int e, float2 &x, float2 &y, float2 &z) {
+        const float k1 = wavenumber(e, N), k1d = wavenumber_d1(e, N);
+        mul_point<OP>(x, y, z, k1, k1d, k2, k2d, k3, k3d, sp);
+    };
+    if constexpr (P::P2) {
+        constexpr int I = 16 / G;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+                float2 b[G];
+#pragma unroll
+                for (int m = 0; m < G; ++m) b[m] = sm[c * CS + (j + G * i + 17 * m) * TL + l];
+                reg_step2<N, -1>(b, j + G * i, w);
+#pragma unroll
+                for (int m = 0; m < G; ++m) a[c][i + I * m] = b[m];
+            }
+#pragma unroll
+        for (int r = 0; r < 16; ++r) mul(j + G * r, a[0][r], a[1][r], a[2][r]);
+    } else {
+        float2 b[3][G];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int m = 0; m < G; ++m) b[c][m] = sm[c * CS + (j + 17 * m) * TL + l];
+            reg_step2<N, -1>(b[c], j, w);
+        }
+#pragma unroll
+        for (int m = 0; m < G; ++m) mul(j + 16 * m, b[0][m], b[1][m], b[2][m]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int m = 0; m < G; ++m) sm[c * CS + (j + 17 * m) * TL + l] = b[c][m];
+        __syncthreads();
+        if (act) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    const int e = j + G * r;
+                    a[c][r] = sm[c * CS + (e + e / 16) * TL + l];
+                }
+        }
+    }
+    if (act) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dft<16>(a[c], 1.f);
+    }
+    __syncthreads();  // the forward results are read
+    if (act) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int r = 0; r < 16; ++r) sm[c * CS + (17 * j + r) * TL + l] = a[c][r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int i = 0; i < 16 / P::TPL; ++i) {
+            const int k = j + P::TPL * i;
+            float2 b[G];
+#pragma unroll
+            for (int m = 0; m < G; ++m) b[m] = sm[c * CS + (k + 17 * m) * TL + l];
+            reg_step2<N, 1>(b, k, w);
+            if (ok) {
+#pragma unroll
+                for (int m = 0; m < G; ++m) base[c * q.cstride + (k + 16 * m) * q.estride] = b[m];
+            }
+        }
+}
+
 // -------------------------------------------------------------- launchers --
 }  // namespace
 
@@ -589,7 +882,10 @@ template <int N, typename TI>
 void r2c_n(const Dims &d, const FftPlan &p, const TI *in, float2 *out, int ncomp,
            cudaStream_t st) {
     const long long nlines = (long long)ncomp * d.n1 * d.n2;
-    if constexpr (N > 0) {
+    if constexpr (fft_reg(N)) {
+        constexpr int TL = RegTile<N>::TL;
+        kr_r2c<N><<<(unsigned)((nlines + 2 * TL - 1) / (2 * TL)), RegTile<N>::T, 0, st>>>(in, out, p.tw, nlines, d.p3);
+    } else if constexpr (N > 0) {
         r2c_l<N, lines_x3(N)>(d, p, in, out, nlines, st);
     } else {
         switch (lines_x3(d.n3)) {
@@ -631,9 +927,24 @@ void c2c_ip(const Dims &d, const FftPlan &p, float2 *data, int ncomp, float s, c
                                                                                   nitems);
 }
 
+// register-resident transform of the lines of a spectrum along x2 or x1
+template <int N, int S>
+void c2c_reg(const FftPlan &p, float2 *data, const RegLines &q, float s, float scale, cudaStream_t st) {
+    constexpr int TL = RegTile<N>::TL;
+    kr_c2c<N, S><<<(q.nlines + TL - 1) / TL, RegTile<N>::T, 0, st>>>(data, p.tw, q, s, scale);
+}
+inline RegLines lines_x2(const Dims &d, int ncomp) {
+    return RegLines{d.p3, (long long)d.n2 * d.p3, (long long)d.n1 * d.n2 * d.p3, d.n1, d.p3, d.h3, ncomp * d.n1 * d.p3};
+}
+inline RegLines lines_x1(const Dims &d, int ncomp) {
+    return RegLines{(long long)d.n2 * d.p3, d.p3, (long long)d.n1 * d.n2 * d.p3, d.n2, d.p3, d.h3, ncomp * d.n2 * d.p3};
+}
+
 template <int N>
 void c2c_n(const Dims &d, const FftPlan &p, float2 *data, int ncomp, float s, cudaStream_t st) {
-    if constexpr (fft_in_place(N)) {
+    if constexpr (fft_reg(N)) {
+        c2c_reg<N, 0>(p, data, lines_x2(d, ncomp), s, 1.f, st);
+    } else if constexpr (fft_in_place(N)) {
         c2c_ip<N, tile_cols(N, 1)>(d, p, data, ncomp, s, st);
     } else if constexpr (N > 0) {
         c2c_t<N, tile_cols(N, 2)>(d, p, data, ncomp, s, st);
@@ -681,7 +992,16 @@ void mul_ip(const Dims &d, const FftPlan &p, float2 *data, const SpecParams &sp,
 template <int N, int OP>
 void mul_n(const Dims &d, const FftPlan &p, float2 *data, const SpecParams &sp, cudaStream_t st) {
     constexpr int NB = 6;  // three component tiles for the current item, three for the next
-    if constexpr (fft_in_place(N)) {
+    if constexpr (fft_reg(N) && OP == OP_X1FWD) {
+        c2c_reg<N, -1>(p, data, lines_x1(d, 3), -1.f, 1.f, st);
+    } else if constexpr (fft_reg(N) && OP == OP_X1INV) {
+        c2c_reg<N, 1>(p, data, lines_x1(d, 3), 1.f, sp.scale, st);
+    } else if constexpr (fft_reg(N)) {
+        constexpr int TL = RegMul<N>::TL;
+        const RegLines q = lines_x1(d, 1);
+        set_smem<kr_mul<N, OP>>(RegMul<N>::smem);
+        kr_mul<N, OP><<<(q.nlines + TL - 1) / TL, RegMul<N>::T, RegMul<N>::smem, st>>>(data, p.tw, q, d.n2, d.n3, sp);
+    } else if constexpr (fft_in_place(N)) {
         // six tiles in all (no scratch): the column count of five data tiles and one more
         mul_ip<N, tile_cols(N, NB - 1), OP>(d, p, data, sp, st);
     } else if constexpr (N > 0) {
@@ -742,7 +1062,12 @@ template <int N, typename TO>
 void c2r_n(const Dims &d, const FftPlan &p, const float2 *in, TO *out, const float *add,
            int ncomp, cudaStream_t st) {
     const long long nlines = (long long)ncomp * d.n1 * d.n2;
-    if constexpr (N > 0) {
+    if constexpr (fft_reg(N)) {
+        constexpr int TL = RegTile<N>::TL, T = RegTile<N>::T;
+        const unsigned grid = (unsigned)((nlines + 2 * TL - 1) / (2 * TL));
+        if (add) kr_c2r<N, EPI_ADD><<<grid, T, 0, st>>>(in, out, add, p.tw, nlines, d.p3);
+        else kr_c2r<N, EPI_STORE><<<grid, T, 0, st>>>(in, out, add, p.tw, nlines, d.p3);
+    } else if constexpr (N > 0) {
         c2r_l<N, lines_x3(N)>(d, p, in, out, add, nlines, st);
     } else {
         switch (lines_x3(d.n3)) {

@@ -25,6 +25,10 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 }
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// the same on the paired FP32 instructions (one issue slot for both parts);
+// used where neither operand is a product that the compiler would contract
+__device__ __forceinline__ float2 cadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 // multiply by s*i (s = +-1)
 __device__ __forceinline__ float2 mul_si(float2 a, float s) { return make_float2(-s * a.y, s * a.x); }
 
@@ -33,8 +37,8 @@ template <int R> __device__ __forceinline__ void dft(float2 *a, float s);
 
 template <> __device__ __forceinline__ void dft<2>(float2 *a, float) {
     float2 t = a[1];
-    a[1] = csub(a[0], t);
-    a[0] = cadd(a[0], t);
+    a[1] = csub2(a[0], t);
+    a[0] = cadd2(a[0], t);
 }
 
 template <> __device__ __forceinline__ void dft<3>(float2 *a, float s) {
@@ -48,16 +52,20 @@ template <> __device__ __forceinline__ void dft<3>(float2 *a, float s) {
     a[2] = csub(m, r);
 }
 
-template <> __device__ __forceinline__ void dft<4>(float2 *a, float s) {
-    float2 t0 = cadd(a[0], a[2]);
-    float2 t1 = csub(a[0], a[2]);
-    float2 t2 = cadd(a[1], a[3]);
-    float2 t3 = mul_si(csub(a[1], a[3]), s);
-    a[0] = cadd(t0, t2);
-    a[2] = csub(t0, t2);
+// PACK: the paired additions (the scalar form for a caller whose products the
+// compiler contracts otherwise)
+template <bool PACK>
+__device__ __forceinline__ void dft4(float2 *a, float s) {
+    const float2 t0 = PACK ? cadd2(a[0], a[2]) : cadd(a[0], a[2]);
+    const float2 t1 = PACK ? csub2(a[0], a[2]) : csub(a[0], a[2]);
+    const float2 t2 = PACK ? cadd2(a[1], a[3]) : cadd(a[1], a[3]);
+    const float2 t3 = mul_si(PACK ? csub2(a[1], a[3]) : csub(a[1], a[3]), s);
+    a[0] = PACK ? cadd2(t0, t2) : cadd(t0, t2);
+    a[2] = PACK ? csub2(t0, t2) : csub(t0, t2);
     a[1] = cadd(t1, t3);
     a[3] = csub(t1, t3);
 }
+template <> __device__ __forceinline__ void dft<4>(float2 *a, float s) { dft4<true>(a, s); }
 
 template <> __device__ __forceinline__ void dft<5>(float2 *a, float s) {
     const float c1 = 0.30901699437494742410f;   // cos(2 pi / 5)
@@ -77,12 +85,13 @@ template <> __device__ __forceinline__ void dft<5>(float2 *a, float s) {
     a[3] = csub(b2, e2);
 }
 
-template <> __device__ __forceinline__ void dft<8>(float2 *a, float s) {
+template <bool PACK>
+__device__ __forceinline__ void dft8(float2 *a, float s) {
     const float h = 0.70710678118654752440f;  // cos(pi/4)
     float2 e[4] = {a[0], a[2], a[4], a[6]};
     float2 o[4] = {a[1], a[3], a[5], a[7]};
-    dft<4>(e, s);
-    dft<4>(o, s);
+    dft4<PACK>(e, s);
+    dft4<PACK>(o, s);
     // o_q *= exp(s 2 pi i q / 8)
     o[1] = cmul(o[1], make_float2(h, s * h));
     o[2] = mul_si(o[2], s);
@@ -93,6 +102,7 @@ template <> __device__ __forceinline__ void dft<8>(float2 *a, float s) {
         a[q + 4] = csub(e[q], o[q]);
     }
 }
+template <> __device__ __forceinline__ void dft<8>(float2 *a, float s) { dft8<true>(a, s); }
 
 // 16 = 4 x 4: DFT-4 over r2 for each r1, twiddle exp(s 2 pi i r1 q1 / 16),
 // DFT-4 over r1 for each q1; output index q1 + 4 q2
@@ -321,9 +331,11 @@ __device__ __forceinline__ void fft_ip(float2 *A, const float2 *__restrict__ tw,
     }
 }
 
-// The lengths whose passes use the in-place plan: powers of two from 128 on
-// (radix-16 stages with one or two butterflies a thread, no register spills);
-// the other lengths keep the out-of-place stages with a scratch tile.
+// The lengths whose staged passes use the in-place plan: powers of two from 128
+// on (radix-16 stages with one or two butterflies a thread, no register
+// spills; 32 to 256 take the register-resident passes of fft_reg.cuh, so 512 is
+// the one left); the other lengths keep the out-of-place stages with a scratch
+// tile.
 __host__ __device__ constexpr bool fft_in_place(int n) { return n >= 128 && (n & (n - 1)) == 0; }
 
 // N > 0: compile-time plan of that length; N == 0: the runtime plan p
