@@ -484,8 +484,9 @@ __device__ __forceinline__ void box_copy(const float *__restrict__ src, const Di
     }
 }
 
-// 64-tap tricubic sum from a box position; pairs of rows go through the
-// paired FP32 instructions (FMUL2/FFMA2), the x2 and x1 contractions too
+// 64-tap tricubic sum of one voxel, rows paired; the same operations per voxel
+// as box_cubic2 below
+template <int PITCH>
 __device__ __forceinline__ float box_cubic(const float *p, const float w1[4], const float w2[4], const float w3[4]) {
     const float2 c0 = make_float2(w3[0], w3[0]), c1 = make_float2(w3[1], w3[1]);
     const float2 c2 = make_float2(w3[2], w3[2]), c3 = make_float2(w3[3], w3[3]);
@@ -496,7 +497,7 @@ __device__ __forceinline__ float box_cubic(const float *p, const float w1[4], co
         float2 sr[2];
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
-            const float *q0 = p + (ia * BS2 + 2 * m) * BOX_PITCH, *q1 = q0 + BOX_PITCH;
+            const float *q0 = p + (ia * BS2 + 2 * m) * PITCH, *q1 = q0 + PITCH;
             float2 t = __fmul2_rn(c0, make_float2(q0[0], q1[0]));
             t = __ffma2_rn(c1, make_float2(q0[1], q1[1]), t);
             t = __ffma2_rn(c2, make_float2(q0[2], q1[2]), t);
@@ -522,8 +523,11 @@ __device__ __forceinline__ void lagrange4x2(float2 t, float2 w[4]) {
     w[3] = __fmul2_rn(__fmul2_rn(make_float2(s, s), b), t);
 }
 
-// the tricubic sums of two voxels, voxel x at box position p, voxel y at q;
-// per voxel the same operations in the same order as box_cubic
+// The 64-tap tricubic sums of two voxels, voxel x at box position p, voxel y at
+// q (rows PITCH floats apart), on the paired FP32 instructions (FMUL2/FFMA2).
+// Per voxel: x3 sums of the 16 rows, then rows 0 and 2 and rows 1 and 3 of
+// each plane, the planes, and the two halves.
+template <int PITCH>
 __device__ __forceinline__ float2 box_cubic2(const float *p, const float *q, const float2 w1[4], const float2 w2[4],
                                              const float2 w3[4]) {
     float2 ux = make_float2(0.f, 0.f), uy = ux;
@@ -532,7 +536,7 @@ __device__ __forceinline__ float2 box_cubic2(const float *p, const float *q, con
         float2 s[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int o = (ia * BS2 + j) * BOX_PITCH;
+            const int o = (ia * BS2 + j) * PITCH;
             float2 t = __fmul2_rn(w3[0], make_float2(p[o], q[o]));
             t = __ffma2_rn(w3[1], make_float2(p[o + 1], q[o + 1]), t);
             t = __ffma2_rn(w3[2], make_float2(p[o + 2], q[o + 2]), t);
@@ -569,13 +573,6 @@ __device__ __forceinline__ float box_linear(const float *p, float u1, float u2, 
 template <int MODE> struct SlOcc {
     static constexpr int v = (MODE == SL_ADJACC || MODE == SL_ADJDOT) ? 2 : 3;
 };
-
-// tiles of block b: a contiguous range, so neighbouring tiles (which share
-// halo rows in L2) run on the same block one after the other
-__device__ __forceinline__ void tile_range(int ntiles, int &tbeg, int &tend) {
-    tbeg = (int)((long long)blockIdx.x * ntiles / gridDim.x);
-    tend = (int)((long long)(blockIdx.x + 1) * ntiles / gridDim.x);
-}
 
 // floors inside the clamp of floor_int: a non-finite or huge displacement
 // (clamped to +-1e6 there, while the box path converts floorf directly) sends
@@ -786,7 +783,7 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
                         lagrange4x2(u[0], w1);
                         lagrange4x2(u[1], w2);
                         lagrange4x2(u[2], w3);
-                        acc = box_cubic2(smem + o[0], smem + o[1], w1, w2, w3);
+                        acc = box_cubic2<BOX_PITCH>(smem + o[0], smem + o[1], w1, w2, w3);
                     }
                     if (ok0) sl_epilogue<MODE>(a, id, N, acc.x, ce[t], cx[t], dot);
                     if (ok1) sl_epilogue<MODE>(a, id + plane, N, acc.y, ce[t + 1], cx[t + 1], dot);
@@ -800,181 +797,262 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
 }
 
 // Box entries of every tile of a displacement field (for fields that do not
-// come from the foot-point kernel, which writes them itself): persistent
-// blocks over the tiles, 12 bytes read per voxel.
+// come from the foot-point kernel, which writes them itself): one tile per
+// block, 12 bytes read per voxel.  Persistent blocks that took their tiles in
+// turn waited for each tile's loads and two barriers (63 us at 192^3, where
+// the bytes take 13).
 __global__ void __launch_bounds__(PT3 * PT2)
 k_tile_ranges(const float *__restrict__ disp, Dims d, int4 *__restrict__ tiles) {
     __shared__ int red[PT2][6];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int nb3 = (d.n3 + PT3 - 1) / PT3, nb2 = (d.n2 + PT2 - 1) / PT2, nb1 = (d.n1 + PT1 - 1) / PT1;
+    const int nb3 = (d.n3 + PT3 - 1) / PT3, nb2 = (d.n2 + PT2 - 1) / PT2;
     const long long N = d.N, plane = (long long)d.n2 * d.n3;
-    int tbeg, tend;
-    tile_range(nb3 * nb2 * nb1, tbeg, tend);
-    for (int tile = tbeg; tile < tend; ++tile) {
-        const int t3 = tile % nb3, r = tile / nb3, t2 = r % nb2, t1 = r / nb2;
-        const int i3 = t3 * PT3 + tx, i2 = t2 * PT2 + ty;
-        int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
-        if (i3 < d.n3 && i2 < d.n2) {
-            for (int t = 0; t < PT1 && t1 * PT1 + t < d.n1; ++t) {
-                const long long id = (long long)(t1 * PT1 + t) * plane + (long long)i2 * d.n3 + i3;
+    const int tile = blockIdx.x, t3 = tile % nb3, r = tile / nb3, t2 = r % nb2, t1 = r / nb2;
+    const int i3 = t3 * PT3 + threadIdx.x, i2 = t2 * PT2 + threadIdx.y;
+    int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
+    const int nok = i3 < d.n3 && i2 < d.n2 ? min(PT1, d.n1 - t1 * PT1) : 0;
+    float x[PT1][3];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const int f = floor_int(disp[c * N + id]);
-                    lo[c] = min(lo[c], f);
-                    hi[c] = max(hi[c], f);
-                }
+    for (int t = 0; t < PT1; ++t)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            x[t][c] = t < nok ? disp[c * N + (long long)(t1 * PT1 + t) * plane + (long long)i2 * d.n3 + i3] : 0.f;
+#pragma unroll
+    for (int t = 0; t < PT1; ++t) {
+        if (t < nok) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int f = floor_int(x[t][c]);
+                lo[c] = min(lo[c], f);
+                hi[c] = max(hi[c], f);
             }
         }
-        tile_box_reduce(lo, hi, red, tiles + tile);
-        __syncthreads();
     }
+    tile_box_reduce(lo, hi, red, tiles + tile);
 }
 
 // ---------------------------------------------------------------------------
 // Foot points from shared-memory boxes (cubic interpolation of v at the RK2
-// predictor).  Persistent blocks walk the 32 x 8 x 4 tiles of the SL steps.
-// For each side the block reduces the floor range of its own predictor
-// displacements s dt v(x)/h over the tile, copies the three components of v
-// over that box into shared memory, and sums the 64 taps of all three
-// components with one set of weights: one shared-memory wavefront per tap and
-// warp, where the global-memory gather of a misaligned 32-float row costs two
-// L1 wavefronts.  A tile whose predictor floors span more than the box allows
-// gathers from global memory instead (the decision is uniform per block).
-// The block also reduces, per tile and side, the floor range of what it wrote:
-// the box entry of that tile for the SL steps.
+// predictor), one 32 x 8 x 4 tile of the SL steps and one side per block.  The
+// block reduces the floor range of its own predictor displacements s dt v(x)/h
+// over the tile, copies the three components of v over that box into shared
+// memory, and sums the 64 taps of all three components with one set of
+// weights: one shared-memory wavefront per tap and warp, where the
+// global-memory gather of a misaligned 32-float row costs two L1 wavefronts.  A tile whose predictor
+// floors span more than the box allows gathers from global memory instead (the
+// decision is uniform per block).  The block also reduces the floor range of
+// what it wrote: the box entry of that tile for the SL steps.  The boxes of the
+// three components share rows of 128 floats (40 columns each), so a row still
+// starts on bank 0 and three blocks fit an SM.  Nothing of a tile is pipelined
+// with the next, so a block has one tile and the hardware fills the SMs as
+// blocks end (one share per resident block: 630 against 616 us at 256^3 for the
+// mean of both sides, the factor and one more side, 103 against 90 at 128^3).
+// Against two persistent blocks per SM with 64-float rows per component: one
+// side 790 -> 550 us at 256^3; its 192 taps take 363 us of the shared-memory pipe.
 // ---------------------------------------------------------------------------
-constexpr int FP_OCC = 2;  // resident blocks per SM: three component boxes each
+constexpr int FP_OCC = 3;
+constexpr int FP_COL = 4 * BOX_CH;           // columns of a component
+constexpr int FP_PITCH = 128;                // floats per row of the three components
+constexpr int FP_FLOATS = BOX_ROWS * FP_PITCH;
+static_assert(3 * FP_COL <= FP_PITCH && 3 * BOX_CH <= PT3, "three components share a row, a warp copies one row");
 
-// v at the predictor point i + q by global-memory gathers (tiles whose
-// predictor floors span more than the box).  Not inlined: its registers stay
-// out of the box path's allocation.
-__device__ __noinline__ float3 fp_gather3(const float *__restrict__ v, const Dims &d, int i1, int i2, int i3,
-                                          float q1, float q2, float q3) {
-    Axis4 a1, a2, a3;
-    axis_stencil(i1, q1, d.n1, d.n2 * d.n3, a1);
-    axis_stencil(i2, q2, d.n2, d.n3, a2);
-    axis_stencil(i3, q3, d.n3, 1, a3);
-    return make_float3(gather64(v, a1, a2, a3), gather64(v + d.N, a1, a2, a3), gather64(v + 2 * d.N, a1, a2, a3));
+// boxes of the three components of v (the rows of box_copy): one row per warp
+// and step, 30 lanes with a 16-byte chunk each; otherwise float by float
+__device__ __forceinline__ void fp_box_copy(const float *__restrict__ v, const Dims &d, long long plane, int lo1,
+                                            int lo2, int lo3, float *buf, bool chunked) {
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    int z = ty / BS2, y = ty - z * BS2;
+    float *dst = buf + ty * FP_PITCH;
+    const float *src[4];
+    constexpr int Q = (3 * BS3 + PT3 - 1) / PT3;
+    static_assert(Q <= 4, "columns of three components in four rounds of a warp");
+    if (chunked) {
+        const int c = tx / BOX_CH;
+        src[0] = v + (c < 3 ? c : 0) * d.N + wrap_index((lo3 & ~3) + 4 * (tx - c * BOX_CH), d.n3);
+    } else {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int i = tx + PT3 * q, c = min(i / BS3, 2), col = min(i - c * BS3, BS3 - 1);
+            src[q] = v + c * d.N + wrap_index(lo3 + col, d.n3);
+        }
+    }
+#pragma unroll 1
+    for (int row = ty; row < BOX_ROWS; row += PT2) {
+        const long long o = wrap_index(lo1 + z, d.n1) * plane + (long long)wrap_index(lo2 + y, d.n2) * d.n3;
+        if (chunked) {
+            if (tx < 3 * BOX_CH) cp_async16(dst + 4 * tx, src[0] + o);
+        } else {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int i = tx + PT3 * q;
+                if (i < 3 * BS3) cp_async4(dst + i + (i / BS3) * (FP_COL - BS3), src[q] + o);
+            }
+        }
+        dst += PT2 * FP_PITCH;
+        y += PT2;
+        if (y >= BS2) {
+            y -= BS2;
+            ++z;
+        }
+    }
 }
 
+__device__ __forceinline__ float sel4(const float w[4], int k) {
+    return k == 0 ? w[0] : (k == 1 ? w[1] : (k == 2 ? w[2] : w[3]));
+}
+
+// v at the predictor point i + q by global-memory gathers (tiles whose
+// predictor floors span more than the box).  The row loops stay rolled and the
+// function inlined: an unrolled one costs the box path registers, a called one
+// spills the caller's values there.
+__device__ __forceinline__ void fp_gather3(const float *__restrict__ v, const Dims &d, int i1, int i2, int i3, float q1,
+                                           float q2, float q3, float out[3]) {
+    const int b1 = wrap_index(i1 + floor_int(q1) - 1, d.n1), b2 = wrap_index(i2 + floor_int(q2) - 1, d.n2);
+    const int b3 = wrap_index(i3 + floor_int(q3) - 1, d.n3);
+    float w1[4], w2[4], w3[4];
+    lagrange4(__fsub_rn(q1, (float)floor_int(q1)), w1);
+    lagrange4(__fsub_rn(q2, (float)floor_int(q2)), w2);
+    lagrange4(__fsub_rn(q3, (float)floor_int(q3)), w3);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[c] = 0.f;
+    int a1 = b1;
+#pragma unroll 1
+    for (int i = 0; i < 4; ++i) {
+        float s2[3] = {0.f, 0.f, 0.f};
+        int a2 = b2;
+#pragma unroll 1
+        for (int j = 0; j < 4; ++j) {
+            const float *row = v + ((long long)a1 * d.n2 + a2) * d.n3;
+            const float wj = sel4(w2, j);
+            int x = b3;
+            float s3[3];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const float f = __ldg(row + c * d.N + x);
+                    s3[c] = k == 0 ? w3[0] * f : fmaf(w3[k], f, s3[c]);
+                }
+                x = x + 1 == d.n3 ? 0 : x + 1;
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) s2[c] = fmaf(wj, s3[c], s2[c]);
+            a2 = a2 + 1 == d.n2 ? 0 : a2 + 1;
+        }
+        const float wi = sel4(w1, i);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) out[c] = fmaf(wi, s2[c], out[c]);
+        a1 = a1 + 1 == d.n1 ? 0 : a1 + 1;
+    }
+}
+
+// one tile per block, side blockIdx.y of those wanted
 __global__ void __launch_bounds__(PT3 * PT2, FP_OCC)
 k_footpoints_box(const float *__restrict__ v, float *__restrict__ dispm, float *__restrict__ dispp, Dims d,
                  float dt, float ih1, float ih2, float ih3, int chunked_in, int4 *__restrict__ tiles_m,
                  int4 *__restrict__ tiles_p) {
     extern __shared__ float smem[];
     __shared__ int red[PT2][6];
-    __shared__ int ored[PT2][6];
-    __shared__ int rng[6];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const bool chunked = chunked_in != 0;
-    const int nb3 = (d.n3 + PT3 - 1) / PT3, nb2 = (d.n2 + PT2 - 1) / PT2, nb1 = (d.n1 + PT1 - 1) / PT1;
+    const int nb3 = (d.n3 + PT3 - 1) / PT3, nb2 = (d.n2 + PT2 - 1) / PT2;
     const long long N = d.N, plane = (long long)d.n2 * d.n3;
     const float ih[3] = {ih1, ih2, ih3};
-    int tbeg, tend;
-    tile_range(nb3 * nb2 * nb1, tbeg, tend);
-    for (int tile = tbeg; tile < tend; ++tile) {
-        const int t3 = tile % nb3, r = tile / nb3, t2 = r % nb2, t1 = r / nb2;
-        const int i3 = t3 * PT3 + tx, i2 = t2 * PT2 + ty;
-        const long long id0 = (long long)t1 * PT1 * plane + (long long)i2 * d.n3 + i3;
-        bool ok[PT1];
-        float vx[PT1][3];
+    const int tile = blockIdx.x;
+    const int t3 = tile % nb3, r = tile / nb3, t2 = r % nb2, t1 = r / nb2;
+    const int i3 = t3 * PT3 + tx, i2 = t2 * PT2 + ty;
+    const long long id0 = (long long)t1 * PT1 * plane + (long long)i2 * d.n3 + i3;
+    const int nok = i3 < d.n3 && i2 < d.n2 ? min(PT1, d.n1 - t1 * PT1) : 0;  // this thread's voxels
+    const bool plus = !dispm || blockIdx.y == 1;
+    float *out = plus ? dispp : dispm;
+    const float sdt = plus ? dt : -dt, hs = 0.5f * sdt;
+    // floor range of the predictor displacements over the tile
+    float vx[PT1][3];
 #pragma unroll
-        for (int t = 0; t < PT1; ++t) {
-            ok[t] = i3 < d.n3 && i2 < d.n2 && t1 * PT1 + t < d.n1;
+    for (int t = 0; t < PT1; ++t)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) vx[t][c] = ok[t] ? v[c * N + id0 + t * plane] : 0.f;
-        }
+        for (int c = 0; c < 3; ++c) vx[t][c] = t < nok ? v[c * N + id0 + t * plane] : 0.f;
+    int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            float *out = s == 0 ? dispm : dispp;
-            if (!out) continue;
-            const float sdt = s == 0 ? -dt : dt, hs = 0.5f * sdt;
-            // floor range of the predictor displacements over the tile
-            int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
-#pragma unroll
-            for (int t = 0; t < PT1; ++t) {
-                if (ok[t]) {
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        const int f = floor_int(sdt * vx[t][c] * ih[c]);
-                        lo[c] = min(lo[c], f);
-                        hi[c] = max(hi[c], f);
-                    }
-                }
-            }
+    for (int t = 0; t < PT1; ++t) {
+        if (t < nok) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const int a = __reduce_min_sync(0xffffffffu, lo[c]), b = __reduce_max_sync(0xffffffffu, hi[c]);
-                if (tx == 0) {
-                    red[ty][2 * c] = a;
-                    red[ty][2 * c + 1] = b;
-                }
+                const int f = floor_int(sdt * vx[t][c] * ih[c]);
+                lo[c] = min(lo[c], f);
+                hi[c] = max(hi[c], f);
             }
-            __syncthreads();
-            if (ty == 0 && tx < 6) {
-                int x = red[0][tx];
-                for (int y = 1; y < PT2; ++y) x = (tx & 1) ? max(x, red[y][tx]) : min(x, red[y][tx]);
-                rng[tx] = x;
-            }
-            __syncthreads();
-            const int f0 = rng[0], f1 = rng[2], f2 = rng[4];
-            const bool fits = rng[1] - f0 <= BOX_SPAN && rng[3] - f1 <= BOX_SPAN && rng[5] - f2 <= BOX_SPAN &&
-                              floor_sane(f0, rng[1]) && floor_sane(f1, rng[3]) && floor_sane(f2, rng[5]);
-            if (fits) {
-#pragma unroll 1
-                for (int c = 0; c < 3; ++c)
-                    box_copy(v + c * N, d, plane, t1 * PT1 + f0 - 1, t2 * PT2 + f1 - 1, t3 * PT3 + f2 - 1,
-                             smem + c * BOX_FLOATS, chunked);
-                cp_async_commit();
-                cp_async_wait<0>();
-                __syncthreads();
-            }
-            const int sh = box_shift(t3 * PT3 + f2 - 1, chunked);
-            // floor range of this side's output over the tile: the box entry
-            // of the SL steps that use it
-            int omn[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, omx[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
-#pragma unroll
-            for (int t = 0; t < PT1; ++t) {
-                if (!ok[t]) continue;
-                const float q1 = sdt * vx[t][0] * ih1, q2 = sdt * vx[t][1] * ih2, q3 = sdt * vx[t][2] * ih3;
-                float w[3];
-                if (fits) {
-                    const float fl1 = floorf(q1), fl2 = floorf(q2), fl3 = floorf(q3);
-                    const int b1 = t + (int)fl1 - f0, b2 = ty + (int)fl2 - f1, b3 = tx + (int)fl3 - f2 + sh;
-                    const float *p = smem + (b1 * BS2 + b2) * BOX_PITCH + b3;
-                    float w1[4], w2[4], w3[4];
-                    lagrange4(q1 - fl1, w1);
-                    lagrange4(q2 - fl2, w2);
-                    lagrange4(q3 - fl3, w3);
-                    if (box_origin_ok(b1, b2, b3, box_cols(chunked))) {
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) w[c] = box_cubic(p + c * BOX_FLOATS, w1, w2, w3);
-                    } else {
-                        w[0] = w[1] = w[2] = 0.f;
-                    }
-                } else {
-                    const float3 g = fp_gather3(v, d, t1 * PT1 + t, i2, i3, q1, q2, q3);
-                    w[0] = g.x;
-                    w[1] = g.y;
-                    w[2] = g.z;
-                }
-                const long long id = id0 + t * plane;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float o = hs * (vx[t][c] + w[c]) * ih[c];
-                    out[c * N + id] = o;
-                    const int f = floor_int(o);
-                    omn[c] = min(omn[c], f);
-                    omx[c] = max(omx[c], f);
-                }
-            }
-            // the boxes, rng and ored are rewritten by the next side or tile
-            // only after further barriers, which the first warp reaches after
-            // it has read ored
-            tile_box_reduce(omn, omx, ored, (s == 0 ? tiles_m : tiles_p) + tile);
-            __syncthreads();
         }
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int a = __reduce_min_sync(0xffffffffu, lo[c]), b = __reduce_max_sync(0xffffffffu, hi[c]);
+        if (tx == 0) {
+            red[ty][2 * c] = a;
+            red[ty][2 * c + 1] = b;
+        }
+    }
+    __syncthreads();
+    // every warp reduces the eight rows for itself
+    const int f0 = __reduce_min_sync(0xffffffffu, red[tx % PT2][0]);
+    const int g0 = __reduce_max_sync(0xffffffffu, red[tx % PT2][1]);
+    const int f1 = __reduce_min_sync(0xffffffffu, red[tx % PT2][2]);
+    const int g1 = __reduce_max_sync(0xffffffffu, red[tx % PT2][3]);
+    const int f2 = __reduce_min_sync(0xffffffffu, red[tx % PT2][4]);
+    const int g2 = __reduce_max_sync(0xffffffffu, red[tx % PT2][5]);
+    const bool fits = g0 - f0 <= BOX_SPAN && g1 - f1 <= BOX_SPAN && g2 - f2 <= BOX_SPAN && floor_sane(f0, g0) &&
+                      floor_sane(f1, g1) && floor_sane(f2, g2);
+    // floor range of the output over the tile: the box entry of the SL steps
+    // that use it
+    int omn[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, omx[3] = {-0x7fffffff, -0x7fffffff, -0x7fffffff};
+    auto store = [&](int t, int c, float x, float w) {
+        const float o = hs * (x + w) * ih[c];
+        out[c * N + id0 + t * plane] = o;
+        const int f = floor_int(o);
+        omn[c] = min(omn[c], f);
+        omx[c] = max(omx[c], f);
+    };
+    if (fits) {
+        fp_box_copy(v, d, plane, t1 * PT1 + f0 - 1, t2 * PT2 + f1 - 1, t3 * PT3 + f2 - 1, smem, chunked);
+        cp_async_commit();
+        cp_async_wait<0>();
+    }
+    __syncthreads();  // the boxes have arrived; red is read and may be written again
+    if (fits) {
+        const int sh = box_shift(t3 * PT3 + f2 - 1, chunked);
+        const unsigned e0 = (unsigned)((ty - f0 * BS2 - f1) * FP_PITCH + tx - f2 + sh) -
+                            FLOOR_BITS * (unsigned)(BS2 * FP_PITCH + FP_PITCH + 1);
+#pragma unroll
+        for (int t = 0; t < PT1; ++t) {
+            if (t < nok) {
+                const float q0 = sdt * vx[t][0] * ih1, q1 = sdt * vx[t][1] * ih2, q2 = sdt * vx[t][2] * ih3;
+                const float m0 = __fadd_rd(q0, FLOOR_MAGIC), m1 = __fadd_rd(q1, FLOOR_MAGIC);
+                const float m2 = __fadd_rd(q2, FLOOR_MAGIC);
+                const unsigned b0 = __float_as_uint(m0), b1 = __float_as_uint(m1), b2 = __float_as_uint(m2);
+                const float *p = smem + (e0 + (unsigned)(t * BS2 * FP_PITCH) + b0 * (unsigned)(BS2 * FP_PITCH) +
+                                         b1 * (unsigned)FP_PITCH + b2);
+                const bool in = box_origin_ok(t + (int)(b0 - FLOOR_BITS) - f0, ty + (int)(b1 - FLOOR_BITS) - f1,
+                                              tx + (int)(b2 - FLOOR_BITS) - f2 + sh, box_cols(chunked));
+                float w1[4], w2[4], w3[4];
+                lagrange4(__fsub_rn(q0, m0 - FLOOR_MAGIC), w1);
+                lagrange4(__fsub_rn(q1, m1 - FLOOR_MAGIC), w2);
+                lagrange4(__fsub_rn(q2, m2 - FLOOR_MAGIC), w3);
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    store(t, c, vx[t][c], in ? box_cubic<FP_PITCH>(p + c * FP_COL, w1, w2, w3) : 0.f);
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (int t = 0; t < nok; ++t) {
+            const long long id = id0 + t * plane;
+            const float x[3] = {v[id], v[N + id], v[2 * N + id]};
+            float w[3];
+            fp_gather3(v, d, t1 * PT1 + t, i2, i3, sdt * x[0] * ih1, sdt * x[1] * ih2, sdt * x[2] * ih3, w);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) store(t, c, x[c], w[c]);
+        }
+    }
+    tile_box_reduce(omn, omx, red, (plus ? tiles_p : tiles_m) + tile);
 }
 
 // SM count of the device current at the first call (thread-safe initialisation)
@@ -994,15 +1072,6 @@ template <typename T>
 inline int chunk_ok(const Dims &d, const T *f) {
     const int per = 16 / (int)sizeof(T);
     return (d.n3 % per == 0 && ((uintptr_t)f & 15) == 0) ? 1 : 0;
-}
-
-inline int pipe_blocks(const Dims &d, int per_sm) {
-    const long long ntiles = (long long)((d.n3 + PT3 - 1) / PT3) * ((d.n2 + PT2 - 1) / PT2) *
-                             ((d.n1 + PT1 - 1) / PT1);
-    // at most kReduceBlocks: a dot-product step leaves one partial sum per block
-    long long want = (long long)per_sm * num_sms();
-    if (want > kReduceBlocks) want = kReduceBlocks;
-    return (int)(ntiles < want ? ntiles : want);
 }
 
 // Consecutive tiles per block of an SL step with `slots` resident blocks on
@@ -1126,7 +1195,7 @@ long long tile_count(const Dims &d) {
 
 void launch_tile_ranges(const Dims &d, const float *disp, int4 *tiles, cudaStream_t st, Profiler *prof) {
     ProfScope ps(prof, CLAIRE_K_FOOTPOINT, st, 12.0 * d.N, 1);
-    k_tile_ranges<<<pipe_blocks(d, 4), dim3(PT3, PT2), 0, st>>>(disp, d, tiles);
+    k_tile_ranges<<<(unsigned)tile_count(d), dim3(PT3, PT2), 0, st>>>(disp, d, tiles);
 }
 
 void launch_footpoints(const Dims &d, int nt, const float *v, float *dispm, float *dispp, int4 *tiles_m,
@@ -1146,11 +1215,11 @@ void launch_footpoints(const Dims &d, int nt, const float *v, float *dispm, floa
         return;
     }
     ProfScope ps(prof, CLAIRE_K_FOOTPOINT, st, (double)d.N * (12 + (dispm ? 12 : 0) + (dispp ? 12 : 0)), 1);
-    const size_t smem = 3 * BOX_FLOATS * sizeof(float);
+    const size_t smem = FP_FLOATS * sizeof(float);
     static SmemAttr attr;  // once per device
     attr.ensure(k_footpoints_box, (int)smem, "k_footpoints_box");
-    k_footpoints_box<<<pipe_blocks(d, FP_OCC), dim3(PT3, PT2), smem, st>>>(v, dispm, dispp, d, dt, i1, i2, i3,
-                                                                          chunk_ok(d, v), tiles_m, tiles_p);
+    k_footpoints_box<<<dim3((unsigned)tile_count(d), dispm && dispp ? 2 : 1), dim3(PT3, PT2), smem, st>>>(
+        v, dispm, dispp, d, dt, i1, i2, i3, chunk_ok(d, v), tiles_m, tiles_p);
 }
 
 void launch_interp(const Dims &d, const float *f, const float *disp, float *out, int4 *tiles,
