@@ -83,6 +83,42 @@ void launch_spec_twolevel(const Dims &df, float2 *specf, const Dims &dc, const f
 void launch_grad_fd8(const Dims &d, const float *f, float *g, cudaStream_t st, Profiler *prof);
 void launch_div_fd8(const Dims &d, const float *v, float *out, cudaStream_t st, Profiler *prof);
 
+// lines of a strided transform pass: consecutive columns of consecutive planes
+// (ncol per plane, the first nval of them valid), components of nplane planes
+struct RegLines {
+    long long estride;  // between elements of a line
+    long long pstride;  // between planes
+    long long cstride;  // between components
+    int nplane, ncol, nval;
+    int nlines;
+};
+
+// One transform pass along an axis whose length has a two-step register plan
+// (fft_gen.cuh); false if the length has none.  The lengths are spread over
+// the translation units fft_gen*.cu.
+struct GenPass {
+    enum Kind { C2C, R2C, C2R, MUL_A, MUL_AINV, DERIV_X3, DERIV_STRIDED } kind;
+    const float2 *tw = nullptr;
+    const float *in = nullptr, *add = nullptr;
+    float *out = nullptr;
+    __half *out_h = nullptr;
+    float2 *spec = nullptr;
+    RegLines q{};             // strided passes
+    long long nlines = 0;     // x3 passes
+    int p3 = 0, n2 = 0, n3 = 0, vec = 0;
+    float s = 0.f, scale = 1.f;
+    SpecParams sp{};
+};
+bool gen_pass0(int n, const GenPass &a, cudaStream_t st);
+bool gen_pass1(int n, const GenPass &a, cudaStream_t st);
+bool gen_pass2(int n, const GenPass &a, cudaStream_t st);
+bool gen_pass3(int n, const GenPass &a, cudaStream_t st);
+bool gen_pass4(int n, const GenPass &a, cudaStream_t st);
+inline bool gen_pass(int n, const GenPass &a, cudaStream_t st) {
+    return gen_pass0(n, a, st) || gen_pass1(n, a, st) || gen_pass2(n, a, st) || gen_pass3(n, a, st) ||
+           gen_pass4(n, a, st);
+}
+
 // ------------------------------------------------------------ transport ----
 // Box entries: the SL kernels work on tiles of 32 (x3) x 8 (x2) x 4 (x1)
 // voxels, ordered x3 fastest; a displacement field comes with one int4 per

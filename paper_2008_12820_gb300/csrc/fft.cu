@@ -223,54 +223,6 @@ k_c2c_x2_ip(float2 *__restrict__ data, FftPlan p, int h3, int p3, float s, int n
 }
 
 // ---------------------------------------------------------------- pass 3 ---
-// The x1 pass's pointwise step at wavenumber (k1, k2, k3) for the three
-// components a, b, c of one spectral point (kd = the wavenumber with an even
-// axis's Nyquist index set to 0, used in the divergence penalty):
-//   OP_A     beta |k|^2 I + gamma kd kd^T
-//   OP_AINV  its inverse by Sherman-Morrison (identity at k = 0)
-//   OP_X1INV scale only; OP_X1FWD nothing
-// each times scale (the 1/N of the inverse transform).
-template <int OP>
-__device__ __forceinline__ void mul_point(float2 &pa, float2 &pb, float2 &pc, float k1, float k1d, float k2,
-                                          float k2d, float k3, float k3d, const SpecParams &sp) {
-    if (OP == OP_X1FWD) {
-    } else if (OP == OP_X1INV) {
-        pa = make_float2(pa.x * sp.scale, pa.y * sp.scale);
-        pb = make_float2(pb.x * sp.scale, pb.y * sp.scale);
-        pc = make_float2(pc.x * sp.scale, pc.y * sp.scale);
-    } else {
-        const float2 a = pa, b = pb, c = pc;
-        const float kk = k1 * k1 + k2 * k2 + k3 * k3;
-        const float kd2 = k1d * k1d + k2d * k2d + k3d * k3d;
-        // fused products spelled out: every pass rounds alike
-        const float2 kv = make_float2(__fmaf_rn(k3d, c.x, __fmaf_rn(k1d, a.x, __fmul_rn(k2d, b.x))),
-                                      __fmaf_rn(k3d, c.y, __fmaf_rn(k1d, a.y, __fmul_rn(k2d, b.y))));
-        float diag, coup;
-        if (OP == OP_A) {
-            diag = sp.beta * kk;
-            coup = sp.gamma;
-        } else {
-            if (kk == 0.f) {
-                diag = 1.f;
-                coup = 0.f;
-            } else {
-                const float bk = sp.beta * kk;
-                diag = 1.f / bk;
-                coup = -sp.gamma * diag / (bk + sp.gamma * kd2);
-            }
-        }
-        const float s = sp.scale;
-        auto row = [&](float kd, const float2 &v) {
-            const float ck = __fmul_rn(coup, kd);
-            return make_float2(__fmul_rn(__fmaf_rn(diag, v.x, __fmul_rn(ck, kv.x)), s),
-                               __fmul_rn(__fmaf_rn(diag, v.y, __fmul_rn(ck, kv.y)), s));
-        };
-        pa = row(k1d, a);
-        pb = row(k2d, b);
-        pc = row(k3d, c);
-    }
-}
-
 // x1 forward, multiplier, x1 inverse, in place; all three components at once
 // (the divergence penalty couples them).  Persistent blocks walk the items
 // (TK k3 columns at one k2 index); the three component tiles of the next item
@@ -903,8 +855,18 @@ void r2c_x3(const Dims &d, const FftPlan &p, const TI *in, float2 *out, int ncom
 #define CASE_N(NN) case NN: r2c_n<NN>(d, p, in, out, ncomp, st); return;
         CLAIRE_CT_SIZES(CASE_N)
 #undef CASE_N
-        default: r2c_n<0>(d, p, in, out, ncomp, st);
+        default: break;
     }
+    if constexpr (std::is_same<TI, float>::value) {
+        GenPass a{GenPass::R2C};
+        a.tw = p.tw;
+        a.in = in;
+        a.spec = out;
+        a.nlines = (long long)ncomp * d.n1 * d.n2;
+        a.p3 = d.p3;
+        if (gen_pass(d.n3, a, st)) return;
+    }
+    r2c_n<0>(d, p, in, out, ncomp, st);
 }
 
 template <int N, int TK>
@@ -962,8 +924,14 @@ void c2c_x2(const Dims &d, const FftPlan &p, float2 *data, int ncomp, float s, c
 #define CASE_N(NN) case NN: c2c_n<NN>(d, p, data, ncomp, s, st); return;
         CLAIRE_CT_SIZES(CASE_N)
 #undef CASE_N
-        default: c2c_n<0>(d, p, data, ncomp, s, st);
+        default: break;
     }
+    GenPass a{GenPass::C2C};
+    a.tw = p.tw;
+    a.spec = data;
+    a.q = lines_x2(d, ncomp);
+    a.s = s;
+    if (!gen_pass(d.n2, a, st)) c2c_n<0>(d, p, data, ncomp, s, st);
 }
 
 template <int N, int TK, int OP>
@@ -1022,8 +990,19 @@ void mul_x1_op(const Dims &d, const FftPlan &p, float2 *data, const SpecParams &
 #define CASE_N(NN) case NN: mul_n<NN, OP>(d, p, data, sp, st); return;
         CLAIRE_CT_SIZES(CASE_N)
 #undef CASE_N
-        default: mul_n<0, OP>(d, p, data, sp, st);
+        default: break;
     }
+    const bool both = OP == OP_A || OP == OP_AINV;
+    GenPass a{both ? (OP == OP_A ? GenPass::MUL_A : GenPass::MUL_AINV) : GenPass::C2C};
+    a.tw = p.tw;
+    a.spec = data;
+    a.q = lines_x1(d, both ? 1 : 3);
+    a.n2 = d.n2;
+    a.n3 = d.n3;
+    a.sp = sp;
+    a.s = OP == OP_X1INV ? 1.f : -1.f;
+    a.scale = OP == OP_X1INV ? sp.scale : 1.f;
+    if (!gen_pass(d.n1, a, st)) mul_n<0, OP>(d, p, data, sp, st);
 }
 
 template <int N, int L, typename TO>
@@ -1085,8 +1064,19 @@ void c2r_x3(const Dims &d, const FftPlan &p, const float2 *in, TO *out, const fl
 #define CASE_N(NN) case NN: c2r_n<NN>(d, p, in, out, add, ncomp, st); return;
         CLAIRE_CT_SIZES(CASE_N)
 #undef CASE_N
-        default: c2r_n<0>(d, p, in, out, add, ncomp, st);
+        default: break;
     }
+    if constexpr (std::is_same<TO, float>::value) {
+        GenPass a{GenPass::C2R};
+        a.tw = p.tw;
+        a.spec = const_cast<float2 *>(in);
+        a.out = out;
+        a.add = add;
+        a.nlines = (long long)ncomp * d.n1 * d.n2;
+        a.p3 = d.p3;
+        if (gen_pass(d.n3, a, st)) return;
+    }
+    c2r_n<0>(d, p, in, out, add, ncomp, st);
 }
 
 // ------------------------------------------------------ grid resampling ---

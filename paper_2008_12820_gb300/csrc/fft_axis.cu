@@ -391,28 +391,6 @@ kr_deriv_x3(const float *__restrict__ in, TO *out, const float *add, const float
     }
 }
 
-// pair of adjacent columns i3, i3 + 1 (ok1: the second is inside the row)
-__device__ __forceinline__ float2 ld_pair(const float *p, bool ok0, bool ok1, bool vec) {
-    if (vec) return ok0 ? *reinterpret_cast<const float2 *>(p) : make_float2(0.f, 0.f);
-    return make_float2(ok0 ? p[0] : 0.f, ok1 ? p[1] : 0.f);
-}
-__device__ __forceinline__ void st_pair(float *p, float2 v, bool ok0, bool ok1, bool vec) {
-    if (vec) {
-        if (ok0) *reinterpret_cast<float2 *>(p) = v;
-    } else {
-        if (ok0) p[0] = v.x;
-        if (ok1) p[1] = v.y;
-    }
-}
-__device__ __forceinline__ void st_pair(__half *p, float2 v, bool ok0, bool ok1, bool vec) {
-    if (vec) {
-        if (ok0) *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(v.x, v.y);
-    } else {
-        if (ok0) p[0] = __float2half_rn(v.x);
-        if (ok1) p[1] = __float2half_rn(v.y);
-    }
-}
-
 // lines along x2 or x1: adjacent x3 columns paired into one complex column.
 // q counts pairs (ncol per row); vec: rows of whole, aligned pairs
 template <int N, int EPI, typename TO>
@@ -458,6 +436,17 @@ kr_deriv_strided(const float *__restrict__ in, TO *out, const float *add, const 
             st_pair(out + off + (k + 16 * m) * q.estride, a[m], ok0, ok1, vec);
         }
     }
+}
+
+// lines of a strided derivative in pairs of x3 columns, and whether the rows
+// are whole, aligned pairs
+template <typename TO>
+RegLines pair_lines(const Dims &d, long long estride, long long pstride, int nplanes, const float *in, TO *out,
+                    const float *add, int &vec) {
+    const int ncol = (d.n3 + 1) / 2;
+    vec = d.n3 % 2 == 0 && ((uintptr_t)in & 7) == 0 && ((uintptr_t)out & (2 * sizeof(TO) - 1)) == 0 &&
+          ((uintptr_t)add & 7) == 0;
+    return RegLines{estride, pstride, 0, nplanes, ncol, ncol, nplanes * ncol};
 }
 
 // ---- axis derivatives: launchers ------------------------------------------
@@ -584,11 +573,9 @@ void deriv_strided_n(const Dims &d, const FftPlan &p, int n, const float *in, TO
                      long long estride, long long pstride, int nplanes, cudaStream_t st) {
     if constexpr (fft_reg(N)) {
         constexpr int TL = RegTile<N>::TL, T = RegTile<N>::T;
-        const int ncol = (d.n3 + 1) / 2;
-        const RegLines q{estride, pstride, 0, nplanes, ncol, ncol, nplanes * ncol};
+        int vec;
+        const RegLines q = pair_lines(d, estride, pstride, nplanes, in, out, add, vec);
         const int grid = (q.nlines + TL - 1) / TL;
-        const int vec = d.n3 % 2 == 0 && ((uintptr_t)in & 7) == 0 && ((uintptr_t)out & (2 * sizeof(TO) - 1)) == 0 &&
-                        ((uintptr_t)add & 7) == 0;
         if constexpr (std::is_same<TO, float>::value) {
             if (add) {
                 kr_deriv_strided<N, EPI_ADD, TO><<<grid, T, 0, st>>>(in, out, add, p.tw, q, d.n3, vec);
@@ -607,6 +594,24 @@ void deriv_strided_n(const Dims &d, const FftPlan &p, int n, const float *in, TO
     }
 }
 
+template <typename TO>
+bool deriv_gen(const Dims &d, const FftPlan *ax, int axis, const float *in, TO *out, const float *add,
+               cudaStream_t st) {
+    const long long plane = (long long)d.n2 * d.n3;
+    GenPass a{axis == 2 ? GenPass::DERIV_X3 : GenPass::DERIV_STRIDED};
+    a.tw = ax[axis].tw;
+    a.in = in;
+    a.add = add;
+    if constexpr (std::is_same<TO, float>::value) a.out = out;
+    else a.out_h = out;
+    a.nlines = (long long)d.n1 * d.n2;
+    a.n3 = d.n3;
+    if (axis < 2)
+        a.q = pair_lines(d, axis == 1 ? d.n3 : plane, axis == 1 ? plane : d.n3, axis == 1 ? d.n1 : d.n2, in, out, add,
+                         a.vec);
+    return gen_pass(axis == 2 ? d.n3 : axis == 1 ? d.n2 : d.n1, a, st);
+}
+
 // d/dx_a of in into out (+ add when given); a = 0, 1, 2 for x1, x2, x3
 template <typename TO>
 void deriv_axis(const Dims &d, const FftPlan *ax, int a, const float *in, TO *out, const float *add,
@@ -617,21 +622,26 @@ void deriv_axis(const Dims &d, const FftPlan *ax, int a, const float *in, TO *ou
 #define CASE_N(NN) case NN: deriv_x3_n<NN>(d, ax[2], in, out, add, st); return;
             CLAIRE_CT_SIZES(CASE_N)
 #undef CASE_N
-            default: deriv_x3_n<0>(d, ax[2], in, out, add, st);
+            default:
+                if (!deriv_gen(d, ax, 2, in, out, add, st)) deriv_x3_n<0>(d, ax[2], in, out, add, st);
         }
     } else if (a == 1) {
         switch (d.n2) {
 #define CASE_N(NN) case NN: deriv_strided_n<NN>(d, ax[1], d.n2, in, out, add, d.n3, plane, d.n1, st); return;
             CLAIRE_CT_SIZES(CASE_N)
 #undef CASE_N
-            default: deriv_strided_n<0>(d, ax[1], d.n2, in, out, add, d.n3, plane, d.n1, st);
+            default:
+                if (!deriv_gen(d, ax, 1, in, out, add, st))
+                    deriv_strided_n<0>(d, ax[1], d.n2, in, out, add, d.n3, plane, d.n1, st);
         }
     } else {
         switch (d.n1) {
 #define CASE_N(NN) case NN: deriv_strided_n<NN>(d, ax[0], d.n1, in, out, add, plane, d.n3, d.n2, st); return;
             CLAIRE_CT_SIZES(CASE_N)
 #undef CASE_N
-            default: deriv_strided_n<0>(d, ax[0], d.n1, in, out, add, plane, d.n3, d.n2, st);
+            default:
+                if (!deriv_gen(d, ax, 0, in, out, add, st))
+                    deriv_strided_n<0>(d, ax[0], d.n1, in, out, add, plane, d.n3, d.n2, st);
         }
     }
 }

@@ -121,15 +121,7 @@ struct RegTile {
     static constexpr int T = RegPlan<N>::TPL * TL;
 };
 
-// position of a block's line `line` (consecutive columns of consecutive
-// planes): columns per plane ncol, valid ones nval
-struct RegLines {
-    long long estride;         // between elements of a line
-    long long pstride;         // between planes
-    long long cstride;         // between components of nplane planes each
-    int nplane, ncol, nval;
-    int nlines;
-};
+// position of a block's line: offset of its plane and column within the row
 __device__ __forceinline__ bool reg_line(const RegLines &q, int line, long long &off, int &col) {
     const int plane = line / q.ncol;
     col = line - plane * q.ncol;
@@ -187,6 +179,76 @@ __device__ __forceinline__ void reg_middle(float2 *sm, const float2 *w, int j, c
         for (int r = 0; r < 16; ++r) sm[at(16 * j + r)] = a[r];
     }
     __syncthreads();
+}
+
+// The x1 pass's pointwise step at wavenumber (k1, k2, k3) for the three
+// components a, b, c of one spectral point (kd = the wavenumber with an even
+// axis's Nyquist index set to 0, used in the divergence penalty):
+//   OP_A     beta |k|^2 I + gamma kd kd^T
+//   OP_AINV  its inverse by Sherman-Morrison (identity at k = 0)
+//   OP_X1INV scale only; OP_X1FWD nothing
+// each times scale (the 1/N of the inverse transform).
+template <int OP>
+__device__ __forceinline__ void mul_point(float2 &pa, float2 &pb, float2 &pc, float k1, float k1d, float k2,
+                                          float k2d, float k3, float k3d, const SpecParams &sp) {
+    if (OP == OP_X1FWD) {
+    } else if (OP == OP_X1INV) {
+        pa = make_float2(pa.x * sp.scale, pa.y * sp.scale);
+        pb = make_float2(pb.x * sp.scale, pb.y * sp.scale);
+        pc = make_float2(pc.x * sp.scale, pc.y * sp.scale);
+    } else {
+        const float2 a = pa, b = pb, c = pc;
+        const float kk = k1 * k1 + k2 * k2 + k3 * k3;
+        const float kd2 = k1d * k1d + k2d * k2d + k3d * k3d;
+        // fused products spelled out: every pass rounds alike
+        const float2 kv = make_float2(__fmaf_rn(k3d, c.x, __fmaf_rn(k1d, a.x, __fmul_rn(k2d, b.x))),
+                                      __fmaf_rn(k3d, c.y, __fmaf_rn(k1d, a.y, __fmul_rn(k2d, b.y))));
+        float diag, coup;
+        if (OP == OP_A) {
+            diag = sp.beta * kk;
+            coup = sp.gamma;
+        } else {
+            if (kk == 0.f) {
+                diag = 1.f;
+                coup = 0.f;
+            } else {
+                const float bk = sp.beta * kk;
+                diag = 1.f / bk;
+                coup = -sp.gamma * diag / (bk + sp.gamma * kd2);
+            }
+        }
+        const float s = sp.scale;
+        auto row = [&](float kd, const float2 &v) {
+            const float ck = __fmul_rn(coup, kd);
+            return make_float2(__fmul_rn(__fmaf_rn(diag, v.x, __fmul_rn(ck, kv.x)), s),
+                               __fmul_rn(__fmaf_rn(diag, v.y, __fmul_rn(ck, kv.y)), s));
+        };
+        pa = row(k1d, a);
+        pb = row(k2d, b);
+        pc = row(k3d, c);
+    }
+}
+
+// pair of adjacent columns i3, i3 + 1 (ok1: the second is inside the row)
+__device__ __forceinline__ float2 ld_pair(const float *p, bool ok0, bool ok1, bool vec) {
+    if (vec) return ok0 ? *reinterpret_cast<const float2 *>(p) : make_float2(0.f, 0.f);
+    return make_float2(ok0 ? p[0] : 0.f, ok1 ? p[1] : 0.f);
+}
+__device__ __forceinline__ void st_pair(float *p, float2 v, bool ok0, bool ok1, bool vec) {
+    if (vec) {
+        if (ok0) *reinterpret_cast<float2 *>(p) = v;
+    } else {
+        if (ok0) p[0] = v.x;
+        if (ok1) p[1] = v.y;
+    }
+}
+__device__ __forceinline__ void st_pair(__half *p, float2 v, bool ok0, bool ok1, bool vec) {
+    if (vec) {
+        if (ok0) *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(v.x, v.y);
+    } else {
+        if (ok0) p[0] = __float2half_rn(v.x);
+        if (ok1) p[1] = __float2half_rn(v.y);
+    }
 }
 
 }  // namespace

@@ -1,7 +1,8 @@
 """The register-resident line transforms (lengths 16 G, G in 2, 4, 6, 8, 10, 12,
-16) against the FP64 oracle: every length along every axis, rows of an odd
-number of columns (no column pairs to load at once), more lines than fill the
-last block, and fields that are only 4-byte aligned."""
+16, and the other products of 2, 3 and 5 from 36 to 240) against the FP64
+oracle: every length along an axis of each kind of pass, rows of an odd number
+of columns (no column pairs to load at once), more lines than fill the last
+block, and fields that are only 4-byte aligned."""
 import numpy as np
 import pytest
 import torch
@@ -36,6 +37,9 @@ def unaligned(a):
 # (x1, x2, x3): each of the seven lengths on each axis
 SHAPES = [(32, 64, 96), (64, 96, 32), (96, 32, 64), (128, 6, 160), (5, 160, 192), (160, 192, 4), (192, 10, 128),
           (4, 128, 256), (256, 5, 15), (6, 256, 27), (160, 9, 25), (32, 96, 45), (128, 64, 9)]
+# two-step plans of other lengths: as x1, x2 and x3 each once
+OTHER = [36, 40, 45, 48, 50, 54, 60, 72, 75, 80, 90, 100, 108, 120, 135, 144, 150, 180, 200, 216, 225, 240]
+SHAPES += [s for n in OTHER for s in ((n, 9, 10), (6, n, 15), (5, 8, n))]
 
 
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
