@@ -501,8 +501,7 @@ struct claire_ctx {
                     cudaGraphConditionalHandle h_tail, int maxit, bool fixed) {
         const long long N = g.d.N, n3 = 3 * N;
         float *ir = work, *iz = ir + n3, *ip = iz + n3, *iq = ip + n3, *iAp = iq + n3;
-        launch_h0_apply(iq, iAp, gm, ip, N, st, &prof);
-        launch_dot(ip, iq, n3, partial, ictl + 2, st, &prof);
+        launch_h0_apply(iq, iAp, gm, ip, N, partial, ictl + 2, st, &prof);
         launch_pcg_update(s, nullptr, ir, ip, iAp, iq, 0.f, N, partial, ictl + 6, st, &prof, false, ictl + 2,
                           ictl + 3, nullptr);
         launch_inner_ctl(ictl, h, h_tail, maxit, fixed, st, &prof);
@@ -577,8 +576,8 @@ struct claire_ctx {
         double rz = dot(ir, iz, n3);
         int it = 0;
         while (it < maxit) {
-            launch_h0_apply(iq, iAp, gm, ip, N, st, &prof);
-            const double pq = dot(ip, iq, n3);
+            launch_h0_apply(iq, iAp, gm, ip, N, partial, dres, st, &prof);
+            const double pq = fetch();
             if (!(pq > 0)) break;
             launch_pcg_update(s, nullptr, ir, ip, iAp, iq, (float)(rz / pq), N, partial, slot, st, &prof);
             ++it;
@@ -1242,7 +1241,9 @@ int claire_create_ex(int nx, int ny, int nz, int nt, double beta, double gamma, 
         c->s1b = c->alloc_f(N);
         c->fdisp = c->alloc_f(3 * N);
         c->spec = (float2 *)c->alloc_bytes((size_t)3 * nx * ny * c->d.p3 * sizeof(float2));
-        c->partial = (double *)c->alloc_bytes(4 * kReduceBlocks * sizeof(double));
+        c->partial = (double *)c->alloc_bytes(kPartialDoubles * sizeof(double));
+        CK(cudaMemset(c->partial, 0, kPartialDoubles * sizeof(double)));
+        CK(cudaStreamSynchronize(0));  // before work on any other stream can use it
         c->dres = (double *)c->alloc_bytes(16 * sizeof(double));
         c->dflag = (int *)c->alloc_bytes(sizeof(int));
         c->ntiles = tile_count(c->d);

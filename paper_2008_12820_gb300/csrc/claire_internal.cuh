@@ -201,7 +201,8 @@ void spectral_div_1d(const Dims &d, const FftPlan *ax, const float *v, float *ou
 void launch_grad_fd8(const Dims &d, const float *f, __half *g, cudaStream_t st, Profiler *prof);
 
 // ------------------------------------------------------------- vectors ----
-// FP64 reductions; results land in dev_out[0..k) (device doubles)
+// FP64 reductions; results land in dev_out[0..k) (device doubles).  partial: the
+// context's buffer of kPartialDoubles, zeroed when it is made.
 // dev_out[0] = sum of partial[0..nb) (+ add[0] if add is non-null)
 void launch_finalize(const double *partial, int nb, const double *add, double *dev_out, cudaStream_t st);
 // the four dot products of the line search: dev_out[0..3] = g.x, x.Av, v.Ax, x.Ax
@@ -211,11 +212,6 @@ void launch_dot(const float *a, const float *b, long long n, double *partial, do
                 cudaStream_t st, Profiler *prof);
 void launch_sqdiff(const float *a, const float *b, long long n, double *partial,
                    double *dev_out, cudaStream_t st, Profiler *prof);
-void launch_pcg_xr(float *x, float *r, const float *p, const float *q, float alpha,
-                   long long n, double *partial, double *dev_out, cudaStream_t st,
-                   Profiler *prof);  // x += a p, r -= a q, out = ||r||^2
-void launch_pcg_p(float *p, const float *z, float beta, long long n, cudaStream_t st,
-                  Profiler *prof);   // p = z + beta p
 void launch_axpby(float *out, float a, const float *x, float b, const float *y, long long n,
                   cudaStream_t st, Profiler *prof);  // out = a x + b y
 void launch_diff_flag(const float *a, const float *b, long long n, int *flag, cudaStream_t st,
@@ -264,10 +260,12 @@ void launch_pcg_dir_u0(float *p, float *Ap, const float *z, const float *r, cons
                        float b, long long N, bool init, const __half *gm0, float *u0, float hdt, double *partial,
                        double *pap_out, cudaStream_t st, Profiler *prof, const double *dbn = nullptr,
                        const double *dbd = nullptr);
-// q = Ap + gm (gm . p): the zero-velocity Hessian given beta0*A p
-void launch_h0_apply(float *q, const float *Ap, const float *gm, const float *p, long long N,
-                     cudaStream_t st, Profiler *prof);
+// q = Ap + gm (gm . p): the zero-velocity Hessian given beta0*A p; dev_out[0] =
+// p . q
+void launch_h0_apply(float *q, const float *Ap, const float *gm, const float *p, long long N, double *partial,
+                     double *dev_out, cudaStream_t st, Profiler *prof);
 constexpr int kReduceBlocks = 1216;  // 152 SMs x 8
+constexpr int kPartialDoubles = 4 * kReduceBlocks + 1;  // block partials and the ticket of the last block
 
 // grid of a persistent transform pass: as many blocks as fit the SMs at this
 // shared memory per block (227 KB per SM, 1 KB reserved per block, at most 8

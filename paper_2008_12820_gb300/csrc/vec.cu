@@ -6,8 +6,9 @@
 // transformations in FP32 (Acc2, reduce.cuh), as accurate as summing in twice
 // the working precision; the pair (sum, compensation) is widened to FP64
 // once, a block reduces in FP64 by warp shuffles, block partials go to a
-// fixed-size array, and one block sums them in a fixed order: deterministic
-// for a given grid.
+// fixed-size array, and the block that finishes last sums them in a fixed
+// order: deterministic for a given grid.  (A second kernel for that sum cost
+// 3-4 us a reduction, a tenth of an inner PCG iteration on a 64^3 grid.)
 #include <cuda_fp16.h>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -26,6 +27,32 @@ constexpr int RT = 256;
 
 // block sum of v (1D blocks of RT threads); valid in thread 0
 __device__ __forceinline__ double block_sum(double v) { return block_sum_n<RT>(v, threadIdx.x); }
+
+// One of `ticket` per block, the last one wraps to 0 (ready for the next
+// launch): true in every thread of the block that draws the last one, when the
+// partial sums that each block's thread 0 wrote before are visible to it.
+__device__ __forceinline__ bool last_block(unsigned *ticket) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// the block's sum s (valid in thread 0) into partial; the last block adds the
+// partials up into out[0] (+ add[0] if add is non-null)
+__device__ __forceinline__ void finish_sum(double s, double *partial, double *out, const double *add,
+                                           unsigned *ticket) {
+    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+    if (!last_block(ticket)) return;
+    double t = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += RT) t += __ldcg(partial + i);
+    t = block_sum(t);
+    if (threadIdx.x == 0) out[0] = add ? t + add[0] : t;
+}
 
 // Four consecutive elements at once (16-byte loads and stores) where the
 // length is a multiple of 4 and the pointers are 16-byte aligned: four times
@@ -59,7 +86,8 @@ __device__ __forceinline__ void reduce2_add(Acc2 &acc, float x, float y) {
 
 template <int MODE, typename TA = float, bool V4 = false>
 __global__ void __launch_bounds__(RT) k_reduce2(const TA *__restrict__ a, const float *__restrict__ b,
-                                                long long n, double *__restrict__ partial) {
+                                                long long n, double *__restrict__ partial, double *out,
+                                                unsigned *ticket) {
     Acc2 acc;
     const long long stride = (long long)gridDim.x * RT;
     if (V4) {
@@ -72,8 +100,7 @@ __global__ void __launch_bounds__(RT) k_reduce2(const TA *__restrict__ a, const 
         for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += stride)
             reduce2_add<MODE>(acc, ldv(a + i), b[i]);
     }
-    double s = block_sum(acc.value());
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+    finish_sum(block_sum(acc.value()), partial, out, nullptr, ticket);
 }
 
 __global__ void __launch_bounds__(RT) k_finalize(const double *__restrict__ partial, int nb,
@@ -84,34 +111,22 @@ __global__ void __launch_bounds__(RT) k_finalize(const double *__restrict__ part
     if (threadIdx.x == 0) out[0] = add ? s + add[0] : s;
 }
 
-// x += alpha p ; r -= alpha q ; partial sums of r.r
-__global__ void __launch_bounds__(RT) k_pcg_xr(float *__restrict__ x, float *__restrict__ r,
-                                               const float *__restrict__ p, const float *__restrict__ q,
-                                               float alpha, long long n, double *__restrict__ partial) {
-    Acc2 acc;
-    const long long stride = (long long)gridDim.x * RT;
-    for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += stride) {
-        x[i] = fmaf(alpha, p[i], x[i]);
-        const float ri = fmaf(-alpha, q[i], r[i]);
-        r[i] = ri;
-        acc.add_prod(ri, ri);
-    }
-    double s = block_sum(acc.value());
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(RT) k_pcg_p(float *__restrict__ p, const float *__restrict__ z,
-                                              float beta, long long n) {
-    const long long stride = (long long)gridDim.x * RT;
-    for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += stride)
-        p[i] = fmaf(beta, p[i], z[i]);
-}
-
+template <bool V4>
 __global__ void __launch_bounds__(RT) k_axpby(float *__restrict__ out, float a, const float *__restrict__ x,
                                               float b, const float *__restrict__ y, long long n) {
     const long long stride = (long long)gridDim.x * RT;
-    for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += stride)
-        out[i] = y ? fmaf(a, x[i], b * y[i]) : a * x[i];
+    if (V4) {
+        for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < (n >> 2); i += stride) {
+            float4 xv = ld4(x, i), yv = y ? ld4(y, i) : make_float4(0.f, 0.f, 0.f, 0.f), o;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                lane(o, k) = y ? fmaf(a, lane(xv, k), b * lane(yv, k)) : a * lane(xv, k);
+            st4(out, i, o);
+        }
+    } else {
+        for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += stride)
+            out[i] = y ? fmaf(a, x[i], b * y[i]) : a * x[i];
+    }
 }
 
 __global__ void __launch_bounds__(RT) k_diff_flag(const float *__restrict__ a, const float *__restrict__ b,
@@ -140,19 +155,33 @@ __device__ __forceinline__ void block_sum4(double v[4]) {
     }
 }
 
-// statistics of a vector field r [3][N]: r.r and the sum of each component
-__device__ __forceinline__ void stats_store(Acc2 &rr, Acc2 *sc, double *partial) {
-    double v[4] = {rr.value(), sc[0].value(), sc[1].value(), sc[2].value()};
+// finish_sum for four sums at once (v: this thread's contributions)
+__device__ __forceinline__ void finish_sum4(double v[4], double *partial, double *out, unsigned *ticket) {
     block_sum4(v);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) partial[4 * blockIdx.x + k] = v[k];
     }
+    if (!last_block(ticket)) return;
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += RT)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t[k] += __ldcg(partial + 4 * i + k);
+    block_sum4(t);
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out[k] = t[k];
+}
+
+// statistics of a vector field r [3][N]: r.r and the sum of each component
+__device__ __forceinline__ void stats_store(Acc2 &rr, Acc2 *sc, double *partial, double *out, unsigned *ticket) {
+    double v[4] = {rr.value(), sc[0].value(), sc[1].value(), sc[2].value()};
+    finish_sum4(v, partial, out, ticket);
 }
 
 template <bool V4>
 __global__ void __launch_bounds__(RT) k_stats(const float *__restrict__ r, long long N,
-                                              double *__restrict__ partial) {
+                                              double *__restrict__ partial, double *out, unsigned *ticket) {
     Acc2 rr, sc[3];
     const long long stride = (long long)gridDim.x * RT;
     if (V4) {
@@ -176,7 +205,7 @@ __global__ void __launch_bounds__(RT) k_stats(const float *__restrict__ r, long 
                 sc[c].add(ri, 0.f);
             }
     }
-    stats_store(rr, sc, partial);
+    stats_store(rr, sc, partial, out, ticket);
 }
 
 // PCG update with the regularization term carried along (x, A x, r):
@@ -192,8 +221,8 @@ __global__ void __launch_bounds__(RT) k_pcg_update(float *__restrict__ x, float 
                                                    const float *__restrict__ Ap,
                                                    const float *__restrict__ q, float alpha,
                                                    long long N, double *__restrict__ partial, int q_adds_Ap,
-                                                   const double *__restrict__ dpq, const double *__restrict__ drz,
-                                                   double *__restrict__ pq_out) {
+                                                   const double *dpq, const double *drz, double *pq_out, double *out,
+                                                   unsigned *ticket) {
     Acc2 rr, sc[3];
     const long long stride = (long long)gridDim.x * RT;
     const bool wantAp = Ax || q_adds_Ap;
@@ -247,40 +276,35 @@ __global__ void __launch_bounds__(RT) k_pcg_update(float *__restrict__ x, float 
                 sc[c].add(ri, 0.f);
             }
     }
-    stats_store(rr, sc, partial);
+    stats_store(rr, sc, partial, out, ticket);
 }
 
 // the four line-search dot products in one sweep over g, x, Av, v, Ax
+template <bool V4>
 __global__ void __launch_bounds__(RT) k_ls_dots(const float *__restrict__ g, const float *__restrict__ x,
                                                 const float *__restrict__ Av, const float *__restrict__ v,
                                                 const float *__restrict__ Ax, long long n,
-                                                double *__restrict__ partial) {
+                                                double *__restrict__ partial, double *out, unsigned *ticket) {
     Acc2 a0, a1, a2, a3;
     const long long stride = (long long)gridDim.x * RT;
-    for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += stride) {
-        const float xi = x[i], Axi = Ax[i];
-        a0.add_prod(g[i], xi);
-        a1.add_prod(xi, Av[i]);
-        a2.add_prod(v[i], Axi);
+    auto add = [&](float gi, float xi, float Avi, float vi, float Axi) {
+        a0.add_prod(gi, xi);
+        a1.add_prod(xi, Avi);
+        a2.add_prod(vi, Axi);
         a3.add_prod(xi, Axi);
+    };
+    if (V4) {
+        for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < (n >> 2); i += stride) {
+            float4 gv = ld4(g, i), xv = ld4(x, i), Avv = ld4(Av, i), vv = ld4(v, i), Axv = ld4(Ax, i);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) add(lane(gv, k), lane(xv, k), lane(Avv, k), lane(vv, k), lane(Axv, k));
+        }
+    } else {
+        for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += stride)
+            add(g[i], x[i], Av[i], v[i], Ax[i]);
     }
     double s[4] = {a0.value(), a1.value(), a2.value(), a3.value()};
-    block_sum4(s);
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) partial[4 * blockIdx.x + k] = s[k];
-}
-
-__global__ void __launch_bounds__(RT) k_finalize4(const double *__restrict__ partial, int nb,
-                                                  double *__restrict__ out) {
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < nb; i += RT)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] += partial[4 * i + k];
-    block_sum4(v);
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) out[k] = v[k];
+    finish_sum4(s, partial, out, ticket);
 }
 
 // new search direction and its image under beta*A without an FFT:
@@ -321,11 +345,11 @@ __global__ void __launch_bounds__(RT) k_pcg_dir(float *__restrict__ p, float *__
 template <typename TG, bool V4>
 __global__ void __launch_bounds__(RT, 4) k_pcg_dir_u0(float *__restrict__ p, float *__restrict__ Ap,
                                                    const float *__restrict__ z, const float *__restrict__ r,
-                                                   const double *__restrict__ rsum, const float *__restrict__ Az,
+                                                   const double *rsum, const float *__restrict__ Az,
                                                    float b, long long N, int init, const TG *__restrict__ gm0,
                                                    float *__restrict__ u0, float hdt,
-                                                   double *__restrict__ partial, const double *__restrict__ dbn,
-                                                   const double *__restrict__ dbd) {
+                                                   double *__restrict__ partial, const double *dbn,
+                                                   const double *dbd, double *out, unsigned *ticket) {
     const long long stride = (long long)gridDim.x * RT;
     // dbn, dbd (optional): b = num / den from device memory (the PCG ratio of
     // successive r . z, without a host round trip)
@@ -397,29 +421,63 @@ __global__ void __launch_bounds__(RT, 4) k_pcg_dir_u0(float *__restrict__ p, flo
             u0[i] = hdt * f;
         }
     }
-    if (partial) {
-        const double s = block_sum(pap.value());
-        if (threadIdx.x == 0) partial[blockIdx.x] = s;
-    }
+    if (partial) finish_sum(block_sum(pap.value()), partial, out, nullptr, ticket);
 }
 
-// zero-velocity Hessian applied to p given beta0*A p:  q = Ap + gm (gm . p)
+// zero-velocity Hessian applied to p given beta0*A p, and p . q:
+//   q = Ap + gm (gm . p)
+// (the curvature product rides on the pass that has p and q in registers)
+template <bool V4>
 __global__ void __launch_bounds__(RT) k_h0_apply(float *__restrict__ q, const float *__restrict__ Ap,
                                                  const float *__restrict__ gm, const float *__restrict__ p,
-                                                 long long N) {
+                                                 long long N, double *__restrict__ partial, double *out,
+                                                 unsigned *ticket) {
+    Acc2 pq;
     const long long stride = (long long)gridDim.x * RT;
-    for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < N; i += stride) {
-        const float g1 = gm[i], g2 = gm[N + i], g3 = gm[2 * N + i];
-        const float gp = g1 * p[i] + g2 * p[N + i] + g3 * p[2 * N + i];
-        q[i] = fmaf(g1, gp, Ap[i]);
-        q[N + i] = fmaf(g2, gp, Ap[N + i]);
-        q[2 * N + i] = fmaf(g3, gp, Ap[2 * N + i]);
+    auto voxel = [&](const float g[3], const float pv[3], const float ap[3], float qv[3]) {
+        const float gp = g[0] * pv[0] + g[1] * pv[1] + g[2] * pv[2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            qv[c] = fmaf(g[c], gp, ap[c]);
+            pq.add_prod(pv[c], qv[c]);
+        }
+    };
+    if (V4) {
+        const long long N4 = N >> 2;
+        for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < N4; i += stride) {
+            float4 g4[3], p4[3], a4[3], q4[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                g4[c] = ld4(gm, c * N4 + i);
+                p4[c] = ld4(p, c * N4 + i);
+                a4[c] = ld4(Ap, c * N4 + i);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float g[3] = {lane(g4[0], k), lane(g4[1], k), lane(g4[2], k)};
+                const float pv[3] = {lane(p4[0], k), lane(p4[1], k), lane(p4[2], k)};
+                const float ap[3] = {lane(a4[0], k), lane(a4[1], k), lane(a4[2], k)};
+                float qv[3];
+                voxel(g, pv, ap, qv);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) lane(q4[c], k) = qv[c];
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) st4(q, c * N4 + i, q4[c]);
+        }
+    } else {
+        for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < N; i += stride) {
+            const float g[3] = {gm[i], gm[N + i], gm[2 * N + i]}, pv[3] = {p[i], p[N + i], p[2 * N + i]};
+            const float ap[3] = {Ap[i], Ap[N + i], Ap[2 * N + i]};
+            float qv[3];
+            voxel(g, pv, ap, qv);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) q[c * N + i] = qv[c];
+        }
     }
+    finish_sum(block_sum(pq.value()), partial, out, nullptr, ticket);
 }
 
-// Body force of the Hessian matvec plus the carried beta*A p, and p . q:
-//   q_d = Ap_d + dt sum_j w_j l^j d_d m^j,   partial sums of sum_d p_d q_d
-// (fuses the PCG curvature product into the pass that writes q)
 __global__ void k_f2h(const float *__restrict__ in, __half *__restrict__ out, long long n) {
     for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT)
         out[i] = __float2half_rn(in[i]);
@@ -428,6 +486,10 @@ __global__ void k_h2f(const __half *__restrict__ in, float *__restrict__ out, lo
     for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT)
         out[i] = __half2float(in[i]);
 }
+
+// the ticket of last_block, behind the partial sums (zeroed with the context;
+// launches that share a partial buffer run in order on one stream)
+inline unsigned *ticket_of(double *partial) { return reinterpret_cast<unsigned *>(partial + 4 * kReduceBlocks); }
 
 inline int blocks_for(long long n) {
     long long b = (n + RT - 1) / RT;
@@ -450,30 +512,29 @@ void launch_finalize(const double *partial, int nb, const double *add, double *d
 
 void launch_ls_dots(const float *g, const float *x, const float *Av, const float *v, const float *Ax, long long n,
                     double *partial, double *dev_out, cudaStream_t st, Profiler *prof) {
-    ProfScope ps(prof, CLAIRE_K_REDUCE, st, 20.0 * n, 2);
-    const int nb = blocks_for(n);
-    k_ls_dots<<<nb, RT, 0, st>>>(g, x, Av, v, Ax, n, partial);
-    k_finalize4<<<1, RT, 0, st>>>(partial, nb, dev_out);
+    ProfScope ps(prof, CLAIRE_K_REDUCE, st, 20.0 * n);
+    const bool v4 = v4_ok(n, g, x, Av, v, Ax);
+    const int nb = blocks_for(v4 ? n / 4 : n);
+    if (v4) k_ls_dots<true><<<nb, RT, 0, st>>>(g, x, Av, v, Ax, n, partial, dev_out, ticket_of(partial));
+    else k_ls_dots<false><<<nb, RT, 0, st>>>(g, x, Av, v, Ax, n, partial, dev_out, ticket_of(partial));
 }
 
 void launch_dot(const float *a, const float *b, long long n, double *partial, double *dev_out,
                 cudaStream_t st, Profiler *prof) {
-    ProfScope ps(prof, CLAIRE_K_REDUCE, st, 8.0 * n, 2);
+    ProfScope ps(prof, CLAIRE_K_REDUCE, st, 8.0 * n);
     const bool v4 = v4_ok(n, a, b);
     const int nb = blocks_for(v4 ? n / 4 : n);
-    if (v4) k_reduce2<0, float, true><<<nb, RT, 0, st>>>(a, b, n, partial);
-    else k_reduce2<0><<<nb, RT, 0, st>>>(a, b, n, partial);
-    k_finalize<<<1, RT, 0, st>>>(partial, nb, dev_out);
+    if (v4) k_reduce2<0, float, true><<<nb, RT, 0, st>>>(a, b, n, partial, dev_out, ticket_of(partial));
+    else k_reduce2<0><<<nb, RT, 0, st>>>(a, b, n, partial, dev_out, ticket_of(partial));
 }
 
 void launch_sqdiff(const float *a, const float *b, long long n, double *partial, double *dev_out,
                    cudaStream_t st, Profiler *prof) {
-    ProfScope ps(prof, CLAIRE_K_REDUCE, st, 8.0 * n, 2);
+    ProfScope ps(prof, CLAIRE_K_REDUCE, st, 8.0 * n);
     const bool v4 = v4_ok(n, a, b);
     const int nb = blocks_for(v4 ? n / 4 : n);
-    if (v4) k_reduce2<1, float, true><<<nb, RT, 0, st>>>(a, b, n, partial);
-    else k_reduce2<1><<<nb, RT, 0, st>>>(a, b, n, partial);
-    k_finalize<<<1, RT, 0, st>>>(partial, nb, dev_out);
+    if (v4) k_reduce2<1, float, true><<<nb, RT, 0, st>>>(a, b, n, partial, dev_out, ticket_of(partial));
+    else k_reduce2<1><<<nb, RT, 0, st>>>(a, b, n, partial, dev_out, ticket_of(partial));
 }
 
 void launch_f2h(const float *in, __half *out, long long n, cudaStream_t st, Profiler *prof) {
@@ -486,24 +547,12 @@ void launch_h2f(const __half *in, float *out, long long n, cudaStream_t st, Prof
     k_h2f<<<blocks_for(n), RT, 0, st>>>(in, out, n);
 }
 
-void launch_pcg_xr(float *x, float *r, const float *p, const float *q, float alpha, long long n,
-                   double *partial, double *dev_out, cudaStream_t st, Profiler *prof) {
-    ProfScope ps(prof, CLAIRE_K_VECTOR, st, 24.0 * n, 2);
-    const int nb = blocks_for(n);
-    k_pcg_xr<<<nb, RT, 0, st>>>(x, r, p, q, alpha, n, partial);
-    k_finalize<<<1, RT, 0, st>>>(partial, nb, dev_out);
-}
-
-void launch_pcg_p(float *p, const float *z, float beta, long long n, cudaStream_t st,
-                  Profiler *prof) {
-    ProfScope ps(prof, CLAIRE_K_VECTOR, st, 12.0 * n);
-    k_pcg_p<<<blocks_for(n), RT, 0, st>>>(p, z, beta, n);
-}
-
 void launch_axpby(float *out, float a, const float *x, float b, const float *y, long long n,
                   cudaStream_t st, Profiler *prof) {
     ProfScope ps(prof, CLAIRE_K_VECTOR, st, (y ? 12.0 : 8.0) * n);
-    k_axpby<<<blocks_for(n), RT, 0, st>>>(out, a, x, b, y, n);
+    const bool v4 = v4_ok(n, out, x, y);
+    if (v4) k_axpby<true><<<blocks_for(n / 4), RT, 0, st>>>(out, a, x, b, y, n);
+    else k_axpby<false><<<blocks_for(n), RT, 0, st>>>(out, a, x, b, y, n);
 }
 
 void launch_diff_flag(const float *a, const float *b, long long n, int *flag, cudaStream_t st,
@@ -515,28 +564,26 @@ void launch_diff_flag(const float *a, const float *b, long long n, int *flag, cu
 
 void launch_stats(const float *r, long long N, double *partial, double *dev_out, cudaStream_t st,
                   Profiler *prof) {
-    ProfScope ps(prof, CLAIRE_K_REDUCE, st, 12.0 * N, 2);
+    ProfScope ps(prof, CLAIRE_K_REDUCE, st, 12.0 * N);
     const bool v4 = v4_ok(N, r);
     const int nb = blocks_for(v4 ? N / 4 : N);
-    if (v4) k_stats<true><<<nb, RT, 0, st>>>(r, N, partial);
-    else k_stats<false><<<nb, RT, 0, st>>>(r, N, partial);
-    k_finalize4<<<1, RT, 0, st>>>(partial, nb, dev_out);
+    if (v4) k_stats<true><<<nb, RT, 0, st>>>(r, N, partial, dev_out, ticket_of(partial));
+    else k_stats<false><<<nb, RT, 0, st>>>(r, N, partial, dev_out, ticket_of(partial));
 }
 
 void launch_pcg_update(float *x, float *Ax, float *r, const float *p, const float *Ap,
                        const float *q, float alpha, long long N, double *partial, double *dev_out,
                        cudaStream_t st, Profiler *prof, bool q_adds_Ap, const double *dpq, const double *drz,
                        double *pq_out) {
-    ProfScope ps(prof, CLAIRE_K_VECTOR, st, 3.0 * N * (Ax ? 36 : 24), 2);
+    ProfScope ps(prof, CLAIRE_K_VECTOR, st, 3.0 * N * (Ax ? 36 : 24));
     const bool v4 = v4_ok(N, x, Ax, r, p, Ap, q);
     const int nb = blocks_for(v4 ? N / 4 : N);
     if (v4)
         k_pcg_update<true><<<nb, RT, 0, st>>>(x, Ax, r, p, Ap, q, alpha, N, partial, q_adds_Ap ? 1 : 0, dpq, drz,
-                                             pq_out);
+                                             pq_out, dev_out, ticket_of(partial));
     else
         k_pcg_update<false><<<nb, RT, 0, st>>>(x, Ax, r, p, Ap, q, alpha, N, partial, q_adds_Ap ? 1 : 0, dpq, drz,
-                                              pq_out);
-    k_finalize4<<<1, RT, 0, st>>>(partial, nb, dev_out);
+                                              pq_out, dev_out, ticket_of(partial));
 }
 
 void launch_pcg_dir(float *p, float *Ap, const float *z, const float *r, const double *rsum,
@@ -671,17 +718,15 @@ template <typename TG>
 static void pcg_dir_u0(float *p, float *Ap, const float *z, const float *r, const double *rsum, const float *Az,
                        float b, long long N, bool init, const TG *gm0, float *u0, float hdt, double *partial,
                        double *pap_out, cudaStream_t st, Profiler *prof, const double *dbn, const double *dbd) {
-    ProfScope ps(prof, CLAIRE_K_VECTOR, st, (double)N * (3.0 * (init ? 16 : 24) + 3 * sizeof(TG) + 4),
-                 pap_out ? 2 : 1);
+    ProfScope ps(prof, CLAIRE_K_VECTOR, st, (double)N * (3.0 * (init ? 16 : 24) + 3 * sizeof(TG) + 4));
     const bool v4 = v4_ok(N, p, Ap, z, r, Az, gm0, u0);
     const int nb = blocks_for(v4 ? N / 4 : N);
     if (v4)
         k_pcg_dir_u0<TG, true><<<nb, RT, 0, st>>>(p, Ap, z, r, rsum, Az, b, N, init ? 1 : 0, gm0, u0, hdt,
-                                                  pap_out ? partial : nullptr, dbn, dbd);
+                                                  pap_out ? partial : nullptr, dbn, dbd, pap_out, ticket_of(partial));
     else
         k_pcg_dir_u0<TG, false><<<nb, RT, 0, st>>>(p, Ap, z, r, rsum, Az, b, N, init ? 1 : 0, gm0, u0, hdt,
-                                                   pap_out ? partial : nullptr, dbn, dbd);
-    if (pap_out) k_finalize<<<1, RT, 0, st>>>(partial, nb, pap_out);
+                                                   pap_out ? partial : nullptr, dbn, dbd, pap_out, ticket_of(partial));
 }
 
 void launch_pcg_dir_u0(float *p, float *Ap, const float *z, const float *r, const double *rsum, const float *Az,
@@ -695,10 +740,13 @@ void launch_pcg_dir_u0(float *p, float *Ap, const float *z, const float *r, cons
     pcg_dir_u0(p, Ap, z, r, rsum, Az, b, N, init, gm0, u0, hdt, partial, pap_out, st, prof, dbn, dbd);
 }
 
-void launch_h0_apply(float *q, const float *Ap, const float *gm, const float *p, long long N,
-                     cudaStream_t st, Profiler *prof) {
+void launch_h0_apply(float *q, const float *Ap, const float *gm, const float *p, long long N, double *partial,
+                     double *dev_out, cudaStream_t st, Profiler *prof) {
     ProfScope ps(prof, CLAIRE_K_VECTOR, st, 48.0 * N);
-    k_h0_apply<<<blocks_for(N), RT, 0, st>>>(q, Ap, gm, p, N);
+    const bool v4 = v4_ok(N, q, Ap, gm, p);
+    const int nb = blocks_for(v4 ? N / 4 : N);
+    if (v4) k_h0_apply<true><<<nb, RT, 0, st>>>(q, Ap, gm, p, N, partial, dev_out, ticket_of(partial));
+    else k_h0_apply<false><<<nb, RT, 0, st>>>(q, Ap, gm, p, N, partial, dev_out, ticket_of(partial));
 }
 
 }  // namespace claire
