@@ -285,7 +285,8 @@ __device__ __forceinline__ float gather_lean(const T *__restrict__ f, const Dims
 // of 266).  What bounds the state step is the shared-memory pipe: 64 tap
 // wavefronts per 32 voxels, 10 more of bank conflicts where floors change
 // inside a warp and 8 of box copies and global accesses take 140 us at 256^3;
-// it runs in 181.  A tile whose floors span more than the box gathers from
+// with every tap read once per voxel it ran in 181, with planes shared
+// (SlShare) in 170.  A tile whose floors span more than the box gathers from
 // global memory instead (the decision is uniform per tile), so a region of
 // large displacements slows only its own tiles.
 // ---------------------------------------------------------------------------
@@ -550,6 +551,47 @@ __device__ __forceinline__ float2 box_cubic2(const float *p, const float *q, con
     return __fadd2_rn(ux, uy);
 }
 
+// box_cubic2 where voxel y's stencil lies exactly one plane behind voxel x's
+// (q = p + a plane): the five planes are read once, 80 loads instead of 128
+template <int PITCH>
+__device__ __forceinline__ float2 box_cubic2_shared(const float *p, const float2 w1[4], const float2 w2[4],
+                                                    const float2 w3[4]) {
+    float2 u[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        // rows h and h + 2 of plane ia (voxel x) and of plane ia + 1 (voxel y)
+        float a0[4], a2[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            a0[k] = p[h * PITCH + k];
+            a2[k] = p[(h + 2) * PITCH + k];
+        }
+#pragma unroll
+        for (int ia = 0; ia < 4; ++ia) {
+            float b0[4], b2[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                b0[k] = p[((ia + 1) * BS2 + h) * PITCH + k];
+                b2[k] = p[((ia + 1) * BS2 + h + 2) * PITCH + k];
+            }
+            float2 s0 = __fmul2_rn(w3[0], make_float2(a0[0], b0[0])), s2 = __fmul2_rn(w3[0], make_float2(a2[0], b2[0]));
+#pragma unroll
+            for (int k = 1; k < 4; ++k) {
+                s0 = __ffma2_rn(w3[k], make_float2(a0[k], b0[k]), s0);
+                s2 = __ffma2_rn(w3[k], make_float2(a2[k], b2[k]), s2);
+            }
+            const float2 t = __ffma2_rn(s2, w2[h + 2], __fmul2_rn(s0, w2[h]));
+            u[h] = ia == 0 ? __fmul2_rn(t, w1[0]) : __ffma2_rn(t, w1[ia], u[h]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                a0[k] = b0[k];
+                a2[k] = b2[k];
+            }
+        }
+    }
+    return __fadd2_rn(u[0], u[1]);
+}
+
 // floor of a displacement whose magnitude is below 2^22 without conversion
 // instructions: adding 1.5 * 2^23 rounded down leaves the floor in the low
 // mantissa bits.  bits(m) = FLOOR_BITS + floor, m - FLOOR_MAGIC = floor.
@@ -572,6 +614,15 @@ __device__ __forceinline__ float box_linear(const float *p, float u1, float u2, 
 // adjoint steps hold nine or twelve inputs a voxel and keep two
 template <int MODE> struct SlOcc {
     static constexpr int v = (MODE == SL_ADJACC || MODE == SL_ADJDOT) ? 2 : 3;
+};
+
+// Steps whose voxel pairs read shared planes once where every pair of a warp
+// allows it: those with few epilogue inputs.  State 181 -> 170 us at 256^3 (no
+// change at 128^3, where fewer warps qualify); the second path costs the steps
+// with more inputs spills (incremental state 225 -> 238, adjoint with body
+// force 234 -> 272).
+template <int MODE> struct SlShare {
+    static constexpr bool v = MODE == SL_PLAIN || MODE == SL_ADJ || MODE == SL_ADJFAC;
 };
 
 // floors inside the clamp of floor_int: a non-finite or huge displacement
@@ -736,7 +787,7 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
             if (!g_cur.w) {
                 const Acc2 td = sl_gather_tile<MODE, ORDER>(a, d, t1, t2, t3);
                 if (MODE == SL_ADJDOT) dot.add(td.s, td.c);
-            } else if (inplane) {
+            } else {
                 // box position of this thread's voxel 0 at floors 0, less the
                 // constant part of the floor bits (unsigned: wraps)
                 const int sh = box_shift(t3 * PT3 + g_cur.z - 1, chunked);
@@ -745,7 +796,8 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
                                     FLOOR_BITS * (unsigned)(BS2 * BOX_PITCH + BOX_PITCH + 1);
 #pragma unroll
                 for (int t = 0; t < PT1; t += 2) {
-                    const bool ok0 = FULL || t1 * PT1 + t < d.n1, ok1 = FULL || t1 * PT1 + t + 1 < d.n1;
+                    const bool ok0 = FULL || (inplane && t1 * PT1 + t < d.n1);
+                    const bool ok1 = FULL || (inplane && t1 * PT1 + t + 1 < d.n1);
                     const long long id = id0 + t * plane;
                     float2 u[3];
                     unsigned o[2];
@@ -774,6 +826,9 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
                                               tx + (int)(f2 - FLOOR_BITS) - g_cur.z + sh, box_cols(chunked));
                     }
                     float2 acc = make_float2(0.f, 0.f);
+                    // every lane votes: those outside the grid stand anywhere
+                    // in the box
+                    const bool shared = ORDER == 3 && SlShare<MODE>::v && __all_sync(0xffffffffu, o[1] - o[0] == BS2 * BOX_PITCH);
                     if (!(in[0] && in[1])) {
                     } else if (ORDER == 1) {
                         acc.x = box_linear(smem + o[0], u[0].x, u[1].x, u[2].x);
@@ -783,7 +838,10 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
                         lagrange4x2(u[0], w1);
                         lagrange4x2(u[1], w2);
                         lagrange4x2(u[2], w3);
-                        acc = box_cubic2<BOX_PITCH>(smem + o[0], smem + o[1], w1, w2, w3);
+                        if (shared)
+                            acc = box_cubic2_shared<BOX_PITCH>(smem + o[0], w1, w2, w3);
+                        else
+                            acc = box_cubic2<BOX_PITCH>(smem + o[0], smem + o[1], w1, w2, w3);
                     }
                     if (ok0) sl_epilogue<MODE>(a, id, N, acc.x, ce[t], cx[t], dot);
                     if (ok1) sl_epilogue<MODE>(a, id + plane, N, acc.y, ce[t + 1], cx[t + 1], dot);
