@@ -117,7 +117,7 @@ int claire_forward(claire_ctx *ctx, const float *v, float *m_final, double *mism
 
 /* Differentiable forward (Eq. 2.1b): m(1) from m0 along the characteristics
  * of v, keeping the state only every checkpoint_stride time steps (and at
- * t = 1); *mismatch = 1/2 ||m(1) - m1||^2_{L2} (nullable; synchronizes).
+ * t = 1); *mismatch = 1/2 ||m(1) - m1||^2_{L2} (nullable; synchronizes if given).
  * m_final: float[N] (nullable).  checkpoint_stride in [1, nt], or 0: chosen
  * from the memory left on the device (and under claire_set_workspace_limit)
  * -- every state kept (stride 1: the backward recomputes nothing) when that
@@ -128,6 +128,13 @@ int claire_forward(claire_ctx *ctx, const float *v, float *m_final, double *mism
  * dominates; keep it when it fits, recompute otherwise). */
 int claire_mismatch_forward(claire_ctx *ctx, const float *v, float *m_final, double *mismatch,
                             int checkpoint_stride);
+
+/* Mismatch of the last claire_mismatch_forward without a synchronization:
+ * writes 1/2 ||m(1) - m1||^2_{L2} to *mismatch, one double in DEVICE memory,
+ * in order on the context's stream (the value claire_mismatch_forward returns
+ * to the host).  CLAIRE_ERR_STATE before the first differentiable forward.  No
+ * counterpart in the paper. */
+int claire_mismatch_device(claire_ctx *ctx, double *mismatch);
 
 /* Checkpoint stride the differentiable form of ctx uses (0 before its first
  * claire_mismatch_forward). */

@@ -26,20 +26,20 @@ class TransportMismatch(torch.autograd.Function):
     @staticmethod
     def forward(ctx, v: torch.Tensor, reg: "claire.Registration", checkpoint_stride: int = 2):
         v = v.detach().contiguous()
-        m1_pred, mis = reg.mismatch_forward(v, checkpoint_stride)
+        # no host synchronization: the caller's loss is enqueued while the
+        # forward runs
+        m1_pred, mis = reg.mismatch_forward_device(v, checkpoint_stride)
         ctx.reg = reg
-        return torch.tensor(mis, dtype=torch.float64, device=v.device), m1_pred
+        return mis, m1_pred
 
     @staticmethod
     def backward(ctx, grad_mis, grad_m1):
         reg = ctx.reg
         gmis = float(grad_mis) if grad_mis is not None else 0.0
-        gm = None
-        if grad_m1 is not None:
-            gm = grad_m1.contiguous().float()
-            if not torch.any(gm != 0):
-                gm = None
+        gm = None if grad_m1 is None else grad_m1.contiguous().float()
+        reg._behind_current()
         grad_v = reg.mismatch_backward(gmis, gm)
+        reg._current_behind()
         return grad_v, None, None
 
 

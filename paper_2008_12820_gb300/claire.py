@@ -38,7 +38,7 @@ EXPORTED = [
     "claire_workspace_bytes", "claire_last_error", "claire_precond_noalloc",
     "claire_precond_h0", "claire_solve_continuation", "claire_set_discretization", "claire_solve_batch",
     "claire_mismatch_forward", "claire_mismatch_backward", "claire_solve_host", "claire_set_workspace_limit",
-    "claire_checkpoint_stride", "claire_check_count",
+    "claire_checkpoint_stride", "claire_check_count", "claire_mismatch_device",
 ]
 
 
@@ -107,6 +107,7 @@ def load(path: str = LIB_PATH):
         "claire_set_discretization": [P, I, I],
         "claire_mismatch_forward": [P, V, V, pd, I],
         "claire_mismatch_backward": [P, D, V, V],
+        "claire_mismatch_device": [P, V],
         "claire_checkpoint_stride": [P, ctypes.POINTER(ctypes.c_int)],
         "claire_check_count": [ctypes.POINTER(ctypes.c_ulonglong), I],
         "claire_solve_continuation": [P, V, D, D, D, ctypes.POINTER(SolveOpts),
@@ -328,6 +329,30 @@ class Registration:
         self._c("claire_mismatch_forward", pv, self._scal(m, "m_final"), ctypes.byref(mis),
                 int(checkpoint_stride))
         return m, mis.value
+
+    def mismatch_forward_device(self, v, checkpoint_stride=2):
+        """mismatch_forward without a host synchronization: (m(1), mismatch) with
+        the mismatch a float64 CUDA scalar.  Both are written on the context's
+        stream; torch's current stream is ordered behind it."""
+        m, mis = self._new(), torch.empty((), dtype=torch.float64, device="cuda")
+        self._behind_current()
+        self._c("claire_mismatch_forward", self._vec(v, "v"), self._scal(m, "m_final"), None, int(checkpoint_stride))
+        self._c("claire_mismatch_device", ctypes.c_void_p(mis.data_ptr()))
+        self._current_behind()
+        return m, mis
+
+    # Ordering between the context's stream and torch's current one, where they
+    # differ: the context's work behind what the caller enqueued, and the
+    # caller's later work (and reuse of freed tensors) behind the context's.
+    def _behind_current(self):
+        cur = torch.cuda.current_stream()
+        if cur != self._stream:
+            self._stream.wait_stream(cur)
+
+    def _current_behind(self):
+        cur = torch.cuda.current_stream()
+        if cur != self._stream:
+            cur.wait_stream(self._stream)
 
     def mismatch_backward(self, grad_mismatch, grad_m_final=None, out=None):
         """Euclidean gradient w.r.t. v of grad_mismatch * mismatch +

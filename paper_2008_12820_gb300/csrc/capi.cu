@@ -987,7 +987,9 @@ struct claire_ctx {
     // forward transport keeping only checkpoints; X-, X+ and c at v kept for
     // the backward; returns the mismatch 1/2 ||m(1) - m1||^2.  stride 0: the
     // stride is chosen from the free memory (auto_stride) at the first call
-    double diff_forward(const float *v, float *m_final, int stride) {
+    // m(1) of the last differentiable forward
+    const float *diff_final() const { return ck + (size_t)ck_slot(nt) * d.N; }
+    double diff_forward(const float *v, float *m_final, int stride, bool want_mismatch = true) {
         if (!have_images) throw Error(CLAIRE_ERR_STATE, "images not set (claire_set_images)");
         if (stride == 0) stride = ck_stride ? ck_stride : auto_stride();
         ensure_ck(stride);
@@ -1011,7 +1013,7 @@ struct claire_ctx {
         const float *mT = ck + (size_t)ck_slot(nt) * N;
         if (m_final) CK(cudaMemcpyAsync(m_final, mT, N * sizeof(float), cudaMemcpyDeviceToDevice, st));
         check_launch("mismatch_forward");
-        return mismatch_of(mT);
+        return want_mismatch ? mismatch_of(mT) : 0.0;
     }
 
     // backward of (mismatch, m(1)) -> v: adjoint from l(1) = gmis (m1 - m(1))
@@ -1027,7 +1029,6 @@ struct claire_ctx {
         float *lam = lam2, *lam_next = lam2 + N;
         launch_adjoint_final(d, lam, m1, ck + (size_t)ck_slot(nt) * N, gm_final, (float)gmis,
                              (float)(1.0 / H3), st, &prof);
-        CK(cudaMemsetAsync(bacc, 0, 3 * N * sizeof(float), st));
         const int nseg = (nt + ck_stride - 1) / ck_stride;
         for (int sgi = nseg - 1; sgi >= 0; --sgi) {
             const int j0 = sgi * ck_stride, j1 = std::min(j0 + ck_stride, nt);
@@ -1044,18 +1045,18 @@ struct claire_ctx {
                     launch_state_step(d, seg_m + (size_t)(j - j0) * N, dispm, rng_m(), seg_m + (size_t)(j + 1 - j0) * N,
                                       st, &prof);
             }
-            // body-force terms of levels j1 .. j0+1 with the adjoint steps
-            // j1 -> j0 (and the level j0 = 0 term at the very end)
-            for (int j = j1; j > j0; --j) {
-                const float w = (j == nt ? 0.5f : 1.f) * dt;
-                grad(state(j), gbuf);
-                launch_bodyforce_acc(d, bacc, lam, gbuf, w, st, &prof);
-                launch_adjoint_step(d, lam, dispp, rng_p(), cfac, lam_next, st, &prof, CLAIRE_K_ADJOINT);
-                float *t = lam; lam = lam_next; lam_next = t;
+            // the body force starts with the term of t = 1; each adjoint step
+            // j -> j - 1 adds the term of the level it reaches (weights dt, and
+            // dt/2 at both ends)
+            if (j1 == nt) {
+                grad(state(nt), gbuf);
+                launch_bodyforce_start(d, bacc, lam, gbuf, 0.5f * dt, st, &prof);
             }
-            if (j0 == 0) {
-                grad(state(0), gbuf);
-                launch_bodyforce_acc(d, bacc, lam, gbuf, 0.5f * dt, st, &prof);
+            for (int j = j1; j > j0; --j) {
+                grad(state(j - 1), gbuf);
+                launch_adjoint_acc(d, lam, dispp, rng_p(), cfac, lam_next, gbuf, bacc, (j == 1 ? 0.5f : 1.f) * dt, false,
+                                   nullptr, partial, nullptr, nullptr, st, &prof, CLAIRE_K_ADJOINT);
+                float *t = lam; lam = lam_next; lam_next = t;
             }
         }
         launch_axpby(grad_v, (float)H3, bacc, 0.f, nullptr, 3 * (long long)N, st, &prof);
@@ -1363,8 +1364,18 @@ int claire_mismatch_forward(claire_ctx *ctx, const float *v, float *m_final, dou
     need(v, "v");
     if (checkpoint_stride < 0 || checkpoint_stride > ctx->nt)
         throw Error(CLAIRE_ERR_ARG, "checkpoint_stride must be in [0, nt] (0: chosen from the free memory)");
-    const double mis = ctx->diff_forward(v, m_final, checkpoint_stride);
+    const double mis = ctx->diff_forward(v, m_final, checkpoint_stride, mismatch != nullptr);
     if (mismatch) *mismatch = mis;
+    API_END(ctx)
+}
+
+int claire_mismatch_device(claire_ctx *ctx, double *mismatch) {
+    API_BEGIN(ctx)
+    need(mismatch, "mismatch");
+    if (!ctx->ck_valid) throw Error(CLAIRE_ERR_STATE, "no differentiable forward at this point");
+    launch_sqdiff(ctx->diff_final(), ctx->m1, ctx->d.N, ctx->partial, ctx->dres, ctx->st, &ctx->prof);
+    launch_scalar_scale(mismatch, 0.5 * ctx->h3(), ctx->dres, ctx->st, &ctx->prof);
+    check_launch("mismatch_device");
     API_END(ctx)
 }
 

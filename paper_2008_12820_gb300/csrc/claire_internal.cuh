@@ -139,9 +139,6 @@ void launch_adjoint_factor(const Dims &d, int nt, const float *divv, const float
 // FP16-storage form
 void launch_state_step(const Dims &d, const float *src, const float *dispm, const int4 *tiles_m,
                        float *dst, cudaStream_t st, Profiler *prof, __half *dst_h = nullptr);
-void launch_adjoint_step(const Dims &d, const float *src, const float *dispp, const int4 *tiles_p,
-                         const float *cfac, float *dst, cudaStream_t st, Profiler *prof, int kclass,
-                         __half *dst_h = nullptr);
 void launch_incstate_init(const Dims &d, float dt, const float *vt, const float *gm0, float *u0,
                           cudaStream_t st, Profiler *prof);
 void launch_incstate_step(const Dims &d, float dt, const float *src, const float *dispm,
@@ -175,9 +172,9 @@ void launch_adjfinal_acc(const Dims &d, const float *m1, const float *m, float *
                          const float *Av, float *g, float w, cudaStream_t st, Profiler *prof);
 void launch_adjfinal_acc(const Dims &d, const float *m1, const float *m, float *l, __half *l_h, const __half *gm,
                          const float *Av, float *g, float w, cudaStream_t st, Profiler *prof);
-// b += w * l * gm
-void launch_bodyforce_acc(const Dims &d, float *b, const float *l, const float *gm, float w,
-                          cudaStream_t st, Profiler *prof);
+// b = w * l * gm
+void launch_bodyforce_start(const Dims &d, float *b, const float *l, const float *gm, float w,
+                            cudaStream_t st, Profiler *prof);
 // l = gmis * (m1 - m) - gm_final * inv_h3 (gm_final nullable)
 void launch_adjoint_final(const Dims &d, float *l, const float *m1, const float *m,
                           const float *gm_final, float gmis, float inv_h3, cudaStream_t st,
@@ -249,6 +246,7 @@ void launch_pcg_negcopy(const double *c, float *x, float *Ax, const float *z, co
                         cudaStream_t st, Profiler *prof);
 void launch_pcg_ctl_init(double *c, double thr, cudaStream_t st, Profiler *prof);
 void launch_scalar_set(double *dst, double v, cudaStream_t st, Profiler *prof);
+void launch_scalar_scale(double *dst, double c, const double *src, cudaStream_t st, Profiler *prof);  // dst = c src
 // launch_pcg_dir that also writes u0 = dt/2 * (-p . gm0) (N floats), the
 // first incremental-state field of the next matvec (hdt = dt/2), and, with
 // pap_out non-null, p . Ap of the new direction into *pap_out

@@ -201,7 +201,7 @@ k_footpoints(const float *__restrict__ v, float *__restrict__ dispm, float *__re
 // SL_ADJACC: adjoint step that adds w l^{j-1} grad m^{j-1} to the body force;
 // SL_ADJDOT: the same, and the block partials of p . b of the finished sum
 // (b . b without p).
-enum SlMode { SL_PLAIN = 0, SL_ADJ = 1, SL_INCSTATE = 2, SL_ADJFAC = 3, SL_INCLAST = 4, SL_ADJACC = 5, SL_ADJDOT = 6 };
+enum SlMode { SL_PLAIN = 0, SL_INCSTATE = 2, SL_ADJFAC = 3, SL_INCLAST = 4, SL_ADJACC = 5, SL_ADJDOT = 6 };
 
 // TS: storage type of the gathered and written field; TG: of grad m
 template <typename TS = float, typename TG = float>
@@ -209,11 +209,11 @@ struct SlArgsT {
     const TS *src;      // field gathered at the foot points
     const float *disp;  // foot point minus grid point, index units, [3][N]
     TS *dst;
-    const float *aux;   // SL_ADJ: c;  SL_ADJFAC: div v on the grid
+    const float *aux;   // SL_ADJACC/SL_ADJDOT: c;  SL_ADJFAC: div v on the grid
     const float *vt;    // SL_INCSTATE: vt [3][N]
     const TG *gm;       // SL_INCSTATE: grad m^{j+1};  SL_ADJACC/SL_ADJDOT: grad m^{j-1}  [3][N]
     float dt;
-    __half *dst_h = nullptr;  // SL_PLAIN / SL_ADJ / SL_ADJACC: optional FP16 copy of dst (stored trajectories)
+    __half *dst_h = nullptr;  // SL_PLAIN / SL_ADJACC: optional FP16 copy of dst (stored trajectories)
     float *dst2 = nullptr;    // SL_INCLAST: mt(1) (optional)
     float *acc = nullptr;     // body force b [3][N]: SL_ADJACC/SL_ADJDOT update it, SL_INCLAST starts it (optional)
     float w = 0.f;            // SL_ADJACC/SL_ADJDOT: trapezoid weight of the new term (dt, dt/2 at j = 0)
@@ -355,10 +355,6 @@ __device__ __forceinline__ void sl_epilogue(const A &a, long long id, long long 
     if (MODE == SL_PLAIN) {
         stf(a.dst + id, val);
         if (a.dst_h) a.dst_h[id] = __float2half_rn(val);
-    } else if (MODE == SL_ADJ) {
-        const float r = e[0] * val;
-        stf(a.dst + id, r);
-        if (a.dst_h) a.dst_h[id] = __float2half_rn(r);
     } else if (MODE == SL_ADJFAC) {
         const float dx = e[0];
         stf(a.dst + id, 1.f + 0.5f * a.dt * (val + dx) + 0.5f * a.dt * a.dt * dx * val);
@@ -392,7 +388,7 @@ __device__ __forceinline__ void sl_epilogue(const A &a, long long id, long long 
 
 template <int MODE, typename A>
 __device__ __forceinline__ void sl_load_epi(const A &a, long long id, long long N, float *e) {
-    if (MODE == SL_ADJ || MODE == SL_ADJFAC || MODE == SL_ADJACC || MODE == SL_ADJDOT) {
+    if (MODE == SL_ADJFAC || MODE == SL_ADJACC || MODE == SL_ADJDOT) {
         e[0] = a.aux[id];
     } else if (MODE == SL_INCSTATE || MODE == SL_INCLAST) {
         e[0] = a.vt[id]; e[1] = a.vt[N + id]; e[2] = a.vt[2 * N + id];
@@ -622,7 +618,7 @@ template <int MODE> struct SlOcc {
 // with more inputs spills (incremental state 225 -> 238, adjoint with body
 // force 234 -> 272).
 template <int MODE> struct SlShare {
-    static constexpr bool v = MODE == SL_PLAIN || MODE == SL_ADJ || MODE == SL_ADJFAC;
+    static constexpr bool v = MODE == SL_PLAIN || MODE == SL_ADJFAC;
 };
 
 // floors inside the clamp of floor_int: a non-finite or huge displacement
@@ -1215,15 +1211,13 @@ __global__ void k_adjfinal_acc(const float *__restrict__ m1, const float *__rest
     }
 }
 
-// b += w * l * gm (three components), the streaming form of the body force
-// used when the state history is recomputed segment by segment
-__global__ void k_bodyforce_acc(float *__restrict__ b, const float *__restrict__ l,
-                                const float *__restrict__ gm, float w, long long N) {
+// b = w * l * gm (three components): the body force's first term
+__global__ void k_bodyforce_start(float *__restrict__ b, const float *__restrict__ l,
+                                  const float *__restrict__ gm, float w, long long N) {
     for (long long i = blockIdx.x * (long long)PT + threadIdx.x; i < N; i += (long long)gridDim.x * PT) {
         const float wl = w * l[i];
-        b[i] = fmaf(wl, gm[i], b[i]);
-        b[N + i] = fmaf(wl, gm[N + i], b[N + i]);
-        b[2 * N + i] = fmaf(wl, gm[2 * N + i], b[2 * N + i]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) b[k * N + i] = wl * gm[k * N + i];
     }
 }
 
@@ -1300,14 +1294,6 @@ void launch_state_step(const Dims &d, const float *src, const float *dispm, cons
     ProfScope ps(prof, CLAIRE_K_STATE, st, (20.0 + (dst_h ? 2 : 0)) * d.N, kSlLaunches);
     SlArgs a{src, dispm, dst, nullptr, nullptr, nullptr, 0.f, dst_h};
     launch_pipe<SL_PLAIN>(d, a, tiles_m, st);
-}
-
-void launch_adjoint_step(const Dims &d, const float *src, const float *dispp, const int4 *tiles_p,
-                         const float *cfac, float *dst, cudaStream_t st, Profiler *prof, int kclass,
-                         __half *dst_h) {
-    ProfScope ps(prof, kclass, st, (24.0 + (dst_h ? 2 : 0)) * d.N, kSlLaunches);
-    SlArgs a{src, dispp, dst, cfac, nullptr, nullptr, 0.f, dst_h};
-    launch_pipe<SL_ADJ>(d, a, tiles_p, st);
 }
 
 namespace {
@@ -1418,10 +1404,10 @@ void launch_adjfinal_acc(const Dims &d, const float *m1, const float *m, float *
     adjfinal_acc(d, m1, m, l, l_h, gm, Av, g, w, st, prof);
 }
 
-void launch_bodyforce_acc(const Dims &d, float *b, const float *l, const float *gm, float w,
-                          cudaStream_t st, Profiler *prof) {
-    ProfScope ps(prof, CLAIRE_K_BODYFORCE, st, 40.0 * d.N);
-    k_bodyforce_acc<<<grid1(d.N), PT, 0, st>>>(b, l, gm, w, d.N);
+void launch_bodyforce_start(const Dims &d, float *b, const float *l, const float *gm, float w,
+                            cudaStream_t st, Profiler *prof) {
+    ProfScope ps(prof, CLAIRE_K_BODYFORCE, st, 28.0 * d.N);
+    k_bodyforce_start<<<grid1(d.N), PT, 0, st>>>(b, l, gm, w, d.N);
 }
 
 void launch_adjoint_final(const Dims &d, float *l, const float *m1, const float *m,

@@ -677,6 +677,9 @@ __global__ void k_pcg_ctl_init(double *c, double thr) {
 __global__ void k_scalar_copy(double *dst, const double *src) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *dst = *src;
 }
+__global__ void k_scalar_scale(double *dst, double c, const double *src) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) *dst = c * *src;
+}
 __global__ void k_scalar_set(double *dst, double v) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *dst = v;
 }
@@ -708,6 +711,10 @@ void launch_pcg_ctl_init(double *c, double thr, cudaStream_t st, Profiler *prof)
 void launch_scalar_copy(double *dst, const double *src, cudaStream_t st, Profiler *prof) {
     ProfScope ps(prof, CLAIRE_K_REDUCE, st);
     k_scalar_copy<<<1, 32, 0, st>>>(dst, src);
+}
+void launch_scalar_scale(double *dst, double c, const double *src, cudaStream_t st, Profiler *prof) {
+    ProfScope ps(prof, CLAIRE_K_VECTOR, st, 16.0);
+    k_scalar_scale<<<1, 32, 0, st>>>(dst, c, src);
 }
 void launch_scalar_set(double *dst, double v, cudaStream_t st, Profiler *prof) {
     ProfScope ps(prof, CLAIRE_K_REDUCE, st);
