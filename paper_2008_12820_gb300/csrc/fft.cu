@@ -789,6 +789,160 @@ kr_mul(float2 *__restrict__ data, const float2 *__restrict__ tw, RegLines q, int
         }
 }
 
+// ------------------------------------------------ whole-plane passes -------
+// x3 and x2 transforms of a square plane (n2 = n3 = N) in one launch, a plane
+// per block, for planes that fit shared memory beside their exchange buffer.
+// On grids this small a pass is a launch and one tile per block, so three
+// launches instead of five count: (beta A)^-1 at 32^3 24.7 -> 16.5 us a call, at
+// 64^3 24.9 -> 20.5, at 96^3 42.5 -> 32.2, at 128x96x96 49 -> 41.  At 128 a plane
+// would leave one block per SM.  The steps are those of kr_r2c, kr_c2c and
+// kr_c2r, bit for bit.
+template <int N>
+struct PlanePlan {
+    using P = RegPlan<N>;
+    static constexpr int H = N / 2 + 1, T = N <= 32 ? 128 : 256;
+    static constexpr int PAIR = N / 2 * P::ROWS, COLS = P::ROWS * H;   // exchange: line pairs, columns
+    static constexpr int X = PAIR > COLS ? PAIR : COLS, S = N * H;     // and the half spectrum of the plane
+    static constexpr size_t smem = (size_t)(X + S + P::W) * sizeof(float2);
+};
+__host__ __device__ constexpr bool plane_fft(int n) { return n == 32 || n == 64 || n == 96; }
+
+template <int N>
+__global__ void __launch_bounds__(PlanePlan<N>::T, 512 / PlanePlan<N>::T)
+kr_plane_fwd(const float *__restrict__ in, float2 *__restrict__ out, const float2 *__restrict__ tw, int p3, float s) {
+    using P = RegPlan<N>;
+    using Q = PlanePlan<N>;
+    constexpr int G = P::G, H = Q::H, T = Q::T;
+    extern __shared__ float2 sm[];
+    float2 *x = sm, *sp = sm + Q::X, *w = sp + Q::S;
+    reg_twiddles<N, T>(w, tw);
+    const float *pl = in + (long long)blockIdx.x * N * N;
+    for (int i = threadIdx.x; i < N / 2 * G; i += T) {
+        const int j = i % G, l = i / G;
+        const float *pa = pl + 2 * l * N + j;
+        float2 a[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) a[r] = make_float2(__ldg(pa + G * r), __ldg(pa + N + G * r));
+        dft<16>(a, -1.f);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) x[l * P::ROWS + 17 * j + r] = a[r];
+    }
+    __syncthreads();
+    // N / 2 line pairs of sixteen threads: whole warps (the shuffles)
+    static_assert(N / 2 * 16 % T == 0, "every thread takes part in every round");
+    for (int i = threadIdx.x; i < N / 2 * 16; i += T) {
+        const int k = i % 16, l = i / 16, src = (threadIdx.x & 16) | ((16 - k) & 15);
+        float2 a[G];
+#pragma unroll
+        for (int m = 0; m < G; ++m) a[m] = x[l * P::ROWS + k + 17 * m];
+        reg_step2<N, -1>(a, k, w);
+        float2 *oa = sp + 2 * l * H + k;
+#pragma unroll
+        for (int m = 0; m <= G / 2; ++m) {
+            const float2 z = a[m];
+            float2 zn;
+            zn.x = __shfl_sync(0xffffffffu, a[G - 1 - m].x, src);
+            zn.y = __shfl_sync(0xffffffffu, a[G - 1 - m].y, src);
+            if (k == 0) zn = a[(G - m) % G];
+            const float2 fa = make_float2(0.5f * (z.x + zn.x), 0.5f * (z.y - zn.y));
+            const float2 fb = make_float2(0.5f * (z.y + zn.y), -0.5f * (z.x - zn.x));
+            if (m < G / 2 || k == 0) {
+                oa[16 * m] = fa;
+                oa[H + 16 * m] = fb;
+            }
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < H * G; i += T) {
+        const int col = i % H, j = i / H;
+        float2 a[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) a[r] = sp[(j + G * r) * H + col];
+        dft<16>(a, s);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) x[(17 * j + r) * H + col] = a[r];
+    }
+    __syncthreads();
+    float2 *po = out + (long long)blockIdx.x * N * p3;
+    for (int i = threadIdx.x; i < H * 16; i += T) {
+        const int col = i % H, k = i / H;
+        float2 a[G];
+#pragma unroll
+        for (int m = 0; m < G; ++m) a[m] = x[(k + 17 * m) * H + col];
+        reg_step2<N, 0>(a, k, w, s);
+#pragma unroll
+        for (int m = 0; m < G; ++m) po[(k + 16 * m) * p3 + col] = a[m];
+    }
+}
+
+template <int N, int EPI>
+__global__ void __launch_bounds__(PlanePlan<N>::T, 512 / PlanePlan<N>::T)
+kr_plane_inv(const float2 *__restrict__ in, float *out, const float *add, const float2 *__restrict__ tw, int p3,
+             float s) {
+    using P = RegPlan<N>;
+    using Q = PlanePlan<N>;
+    constexpr int G = P::G, H = Q::H, T = Q::T;
+    extern __shared__ float2 sm[];
+    float2 *x = sm, *sp = sm + Q::X, *w = sp + Q::S;
+    reg_twiddles<N, T>(w, tw);
+    const float2 *pi = in + (long long)blockIdx.x * N * p3;
+    for (int i = threadIdx.x; i < H * G; i += T) {
+        const int col = i % H, j = i / H;
+        float2 a[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) a[r] = __ldg(pi + (j + G * r) * p3 + col);
+        dft<16>(a, s);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) x[(17 * j + r) * H + col] = a[r];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < H * 16; i += T) {
+        const int col = i % H, k = i / H;
+        float2 a[G];
+#pragma unroll
+        for (int m = 0; m < G; ++m) a[m] = x[(k + 17 * m) * H + col];
+        reg_step2<N, 0>(a, k, w, s);
+#pragma unroll
+        for (int m = 0; m < G; ++m) sp[(k + 16 * m) * H + col] = a[m];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < N / 2 * G; i += T) {
+        const int j = i % G, l = i / G;
+        const float2 *pa = sp + 2 * l * H;
+        float2 a[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const int e = j + G * r;
+            const bool lo = r < 8 || (r == 8 && j == 0);  // e <= N / 2
+            const int k = lo ? e : N - e;
+            float2 fa = pa[k], fb = pa[H + k];
+            if ((r == 0 || r == 8) && j == 0) {
+                fa.y = 0.f;
+                fb.y = 0.f;
+            }
+            a[r] = lo ? make_float2(fa.x - fb.y, fa.y + fb.x) : make_float2(fa.x + fb.y, -fa.y + fb.x);
+        }
+        dft<16>(a, 1.f);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) x[l * P::ROWS + 17 * j + r] = a[r];
+    }
+    __syncthreads();
+    const long long o = (long long)blockIdx.x * N * N;
+    for (int i = threadIdx.x; i < N / 2 * 16; i += T) {
+        const int k = i % 16, l = i / 16;
+        float2 a[G];
+#pragma unroll
+        for (int m = 0; m < G; ++m) a[m] = x[l * P::ROWS + k + 17 * m];
+        reg_step2<N, 1>(a, k, w);
+#pragma unroll
+        for (int m = 0; m < G; ++m) {
+            const long long q = o + 2 * l * N + k + 16 * m;
+            out[q] = EPI == EPI_ADD ? a[m].x + add[q] : a[m].x;
+            out[q + N] = EPI == EPI_ADD ? a[m].y + add[q + N] : a[m].y;
+        }
+    }
+}
+
 // -------------------------------------------------------------- launchers --
 }  // namespace
 
@@ -1079,6 +1233,68 @@ void c2r_x3(const Dims &d, const FftPlan &p, const float2 *in, TO *out, const fl
     c2r_n<0>(d, p, in, out, add, ncomp, st);
 }
 
+// the x3 and x2 transforms of ncomp components in one launch, where planes are
+// square and of a length with a whole-plane pass (false: nothing launched)
+template <int N>
+void plane_fwd(const Dims &d, const FftPlan &p, const float *in, float2 *out, int ncomp, cudaStream_t st) {
+    set_smem<kr_plane_fwd<N>>(PlanePlan<N>::smem);
+    kr_plane_fwd<N><<<ncomp * d.n1, PlanePlan<N>::T, PlanePlan<N>::smem, st>>>(in, out, p.tw, d.p3, -1.f);
+}
+template <int N>
+void plane_inv(const Dims &d, const FftPlan &p, const float2 *in, float *out, const float *add, int ncomp,
+               cudaStream_t st) {
+    if (add) {
+        set_smem<kr_plane_inv<N, EPI_ADD>>(PlanePlan<N>::smem);
+        kr_plane_inv<N, EPI_ADD><<<ncomp * d.n1, PlanePlan<N>::T, PlanePlan<N>::smem, st>>>(in, out, add, p.tw, d.p3, 1.f);
+    } else {
+        set_smem<kr_plane_inv<N, EPI_STORE>>(PlanePlan<N>::smem);
+        kr_plane_inv<N, EPI_STORE><<<ncomp * d.n1, PlanePlan<N>::T, PlanePlan<N>::smem, st>>>(in, out, add, p.tw, d.p3,
+                                                                                            1.f);
+    }
+}
+
+// forward transform along x3 and x2 (real to half spectrum), and back
+void forward_32(const Dims &d, const FftPlan *ax, const float *in, float2 *spec, int ncomp, cudaStream_t st,
+                Profiler *prof) {
+    const double R = 4.0 * d.N, C = 8.0 * d.n1 * d.n2 * d.h3;
+    if (d.n2 == d.n3 && plane_fft(d.n3)) {
+        ProfScope ps(prof, CLAIRE_K_FFT_R2C, st, ncomp * (R + C));
+        switch (d.n3) {
+            case 32: plane_fwd<32>(d, ax[2], in, spec, ncomp, st); return;
+            case 64: plane_fwd<64>(d, ax[2], in, spec, ncomp, st); return;
+            default: plane_fwd<96>(d, ax[2], in, spec, ncomp, st); return;
+        }
+    }
+    {
+        ProfScope ps(prof, CLAIRE_K_FFT_R2C, st, ncomp * (R + C));
+        r2c_x3(d, ax[2], in, spec, ncomp, st);
+    }
+    {
+        ProfScope ps(prof, CLAIRE_K_FFT_C2C, st, ncomp * 2 * C);
+        c2c_x2(d, ax[1], spec, ncomp, -1.f, st);
+    }
+}
+void inverse_23(const Dims &d, const FftPlan *ax, float2 *spec, float *out, const float *add, int ncomp,
+                cudaStream_t st, Profiler *prof) {
+    const double R = 4.0 * d.N, C = 8.0 * d.n1 * d.n2 * d.h3;
+    if (d.n2 == d.n3 && plane_fft(d.n3)) {
+        ProfScope ps(prof, CLAIRE_K_FFT_C2R, st, ncomp * (R + C + (add ? R : 0.0)));
+        switch (d.n3) {
+            case 32: plane_inv<32>(d, ax[2], spec, out, add, ncomp, st); return;
+            case 64: plane_inv<64>(d, ax[2], spec, out, add, ncomp, st); return;
+            default: plane_inv<96>(d, ax[2], spec, out, add, ncomp, st); return;
+        }
+    }
+    {
+        ProfScope ps(prof, CLAIRE_K_FFT_C2C, st, ncomp * 2 * C);
+        c2c_x2(d, ax[1], spec, ncomp, +1.f, st);
+    }
+    {
+        ProfScope ps(prof, CLAIRE_K_FFT_C2R, st, ncomp * (R + C + (add ? R : 0.0)));
+        c2r_x3(d, ax[2], spec, out, add, ncomp, st);
+    }
+}
+
 // ------------------------------------------------------ grid resampling ---
 __device__ __forceinline__ bool in_coarse_band(float k, int nc) { return 2.f * fabsf(k) < (float)nc; }
 __device__ __forceinline__ int index_of(float k, int n) { return k < 0.f ? n + (int)k : (int)k; }
@@ -1155,33 +1371,17 @@ void spectral_apply(const Dims &d, const FftPlan *ax, SpecOp op, const SpecParam
         spectral_div_1d(d, ax, in, out, st, prof);
         return;
     }
-    const int nin = 3, nout = 3;
     // algorithmic bytes: real fields 4 B/voxel, half spectra 8 B per stored mode
-    const double R = 4.0 * d.N, C = 8.0 * d.n1 * d.n2 * d.h3;
+    forward_32(d, ax, in, spec, 3, st, prof);
     {
-        ProfScope ps(prof, CLAIRE_K_FFT_R2C, st, nin * (R + C));
-        r2c_x3(d, ax[2], in, spec, nin, st);
-    }
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_C2C, st, nin * 2 * C);
-        c2c_x2(d, ax[1], spec, nin, -1.f, st);
-    }
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_MUL, st, (nin + nout) * C);
+        ProfScope ps(prof, CLAIRE_K_FFT_MUL, st, 6 * 8.0 * d.n1 * d.n2 * d.h3);
         switch (op) {
             case OP_A: mul_x1_op<OP_A>(d, ax[0], spec, sp, st); break;
             case OP_AINV: mul_x1_op<OP_AINV>(d, ax[0], spec, sp, st); break;
             default: break;
         }
     }
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_C2C, st, nout * 2 * C);
-        c2c_x2(d, ax[1], spec, nout, +1.f, st);
-    }
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_C2R, st, nout * (R + C + (add ? R : 0.0)));
-        c2r_x3(d, ax[2], spec, out, add, nout, st);
-    }
+    inverse_23(d, ax, spec, out, add, 3, st, prof);
 }
 
 }  // namespace claire
@@ -1190,36 +1390,18 @@ namespace claire {
 
 void spectral_forward3(const Dims &d, const FftPlan *ax, const float *in, float2 *spec,
                        cudaStream_t st, Profiler *prof) {
-    const double R = 4.0 * d.N, C = 8.0 * d.n1 * d.n2 * d.h3;
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_R2C, st, 3 * (R + C));
-        r2c_x3(d, ax[2], in, spec, 3, st);
-    }
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_C2C, st, 3 * 2 * C);
-        c2c_x2(d, ax[1], spec, 3, -1.f, st);
-    }
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_MUL, st, 6 * C);
-        mul_x1_op<OP_X1FWD>(d, ax[0], spec, SpecParams{0.f, 0.f, 1.f}, st);
-    }
+    forward_32(d, ax, in, spec, 3, st, prof);
+    ProfScope ps(prof, CLAIRE_K_FFT_MUL, st, 6 * 8.0 * d.n1 * d.n2 * d.h3);
+    mul_x1_op<OP_X1FWD>(d, ax[0], spec, SpecParams{0.f, 0.f, 1.f}, st);
 }
 
 void spectral_inverse3(const Dims &d, const FftPlan *ax, float2 *spec, float *out, float scale,
                        cudaStream_t st, Profiler *prof) {
-    const double R = 4.0 * d.N, C = 8.0 * d.n1 * d.n2 * d.h3;
     {
-        ProfScope ps(prof, CLAIRE_K_FFT_MUL, st, 6 * C);
+        ProfScope ps(prof, CLAIRE_K_FFT_MUL, st, 6 * 8.0 * d.n1 * d.n2 * d.h3);
         mul_x1_op<OP_X1INV>(d, ax[0], spec, SpecParams{0.f, 0.f, scale}, st);
     }
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_C2C, st, 3 * 2 * C);
-        c2c_x2(d, ax[1], spec, 3, +1.f, st);
-    }
-    {
-        ProfScope ps(prof, CLAIRE_K_FFT_C2R, st, 3 * (R + C));
-        c2r_x3(d, ax[2], spec, out, nullptr, 3, st);
-    }
+    inverse_23(d, ax, spec, out, nullptr, 3, st, prof);
 }
 
 void launch_spec_restrict(const Dims &df, const float2 *specf, const Dims &dc, float2 *specc,

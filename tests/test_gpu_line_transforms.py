@@ -37,6 +37,8 @@ def unaligned(a):
 # (x1, x2, x3): each of the seven lengths on each axis
 SHAPES = [(32, 64, 96), (64, 96, 32), (96, 32, 64), (128, 6, 160), (5, 160, 192), (160, 192, 4), (192, 10, 128),
           (4, 128, 256), (256, 5, 15), (6, 256, 27), (160, 9, 25), (32, 96, 45), (128, 64, 9)]
+# square planes whose x3 and x2 transforms share a launch
+SHAPES += [(5, 32, 32), (32, 64, 64), (9, 96, 96)]
 # two-step plans of other lengths: as x1, x2 and x3 each once
 OTHER = [36, 40, 45, 48, 50, 54, 60, 72, 75, 80, 90, 100, 108, 120, 135, 144, 150, 180, 200, 216, 225, 240]
 SHAPES += [s for n in OTHER for s in ((n, 9, 10), (6, n, 15), (5, 8, n))]
