@@ -13,9 +13,12 @@
 //   4. x2 inverse, in place.
 //   5. x3 inverse, half spectrum -> real, two lines per complex transform,
 //      with an optional addend in the epilogue.
-// Each pass stages a tile of whole lines in shared memory and runs a
-// mixed-radix (2, 3, 4, 5) Stockham FFT there: natural-order output, no bit
-// reversal, twiddles from a table computed in double on the host.
+// Lengths 32, 64, 96, 128, 160, 192 and 256 (fft_reg.cuh) and the other products
+// of 2, 3 and 5 from 36 to 240 (fft_gen.cuh) run in registers around one exchange
+// through shared memory.  At the other lengths a pass stages a tile of whole
+// lines in shared memory and runs a mixed-radix Stockham FFT there.  Either way:
+// natural-order output, no bit reversal, twiddles from a table computed in
+// double on the host.
 // Strided passes (x2, x1) load tiles of TK consecutive k3 columns so that
 // every row access is a contiguous 8*TK-byte segment.
 #include <cuda_fp16.h>
