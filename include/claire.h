@@ -87,7 +87,9 @@ int claire_create_ex(int nx, int ny, int nz, int nt, double beta, double gamma, 
 /* Release the context and its device memory (NULL is a no-op). */
 int claire_destroy(claire_ctx *ctx);
 
-/* Order all later work of ctx on `stream` (a cudaStream_t; NULL = legacy). */
+/* Order all later work of ctx on `stream` (a cudaStream_t; NULL = legacy).  The
+ * new stream waits for a reduction that claire_mismatch_device left in flight on
+ * the stream before; ordering anything else behind that stream is the caller's. */
 int claire_set_stream(claire_ctx *ctx, void *stream);
 
 /* Change beta and gamma (same rules as claire_create); drops nothing but the

@@ -165,6 +165,28 @@ struct claire_ctx {
     cudaEvent_t ev_main = nullptr, ev_img = nullptr, ev_vout = nullptr;
     bool img_pending = false;  // the image copies on aux may still be running
     float *vdev = nullptr;
+    // End of the last reduction that a call left in flight on its stream.  The
+    // partial sums and their ticket (last_block) serve every reduction of the
+    // context, and two that overlap would leave the ticket off zero for good, so
+    // claire_set_stream puts the new stream behind it.  (A stream under capture
+    // is left alone on either side: its work runs when the graph is launched,
+    // ordered by whoever launches it.)
+    cudaEvent_t ev_reduce = nullptr;
+    static bool capturing(cudaStream_t s) {
+        cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+        const bool known = cudaStreamIsCapturing(s, &c) == cudaSuccess;
+        if (!known) cudaGetLastError();
+        return !known || c != cudaStreamCaptureStatusNone;
+    }
+    void reduction_in_flight() {
+        if (capturing(st)) return;
+        if (!ev_reduce) CK(cudaEventCreateWithFlags(&ev_reduce, cudaEventDisableTiming));
+        CK(cudaEventRecord(ev_reduce, st));
+    }
+    void move_to(cudaStream_t s) {
+        if (s != st && ev_reduce && !capturing(s)) CK(cudaStreamWaitEvent(s, ev_reduce, 0));
+        st = s;
+    }
     void ensure_aux() {
         if (aux) return;
         CK(cudaStreamCreateWithFlags(&aux, cudaStreamNonBlocking));
@@ -224,6 +246,7 @@ struct claire_ctx {
             cudaEventDestroy(ev_img);
             cudaEventDestroy(ev_vout);
         }
+        if (ev_reduce) cudaEventDestroy(ev_reduce);
         for (void *p : allocs) cudaFree(p);
         for (int a = 0; a < 3; ++a) cudaFree((void *)ax[a].tw);
     }
@@ -1271,7 +1294,7 @@ int claire_destroy(claire_ctx *ctx) {
 
 int claire_set_stream(claire_ctx *ctx, void *stream) {
     API_BEGIN(ctx)
-    ctx->st = (cudaStream_t)stream;
+    ctx->move_to((cudaStream_t)stream);
     API_END(ctx)
 }
 
@@ -1376,6 +1399,7 @@ int claire_mismatch_device(claire_ctx *ctx, double *mismatch) {
     launch_sqdiff(ctx->diff_final(), ctx->m1, ctx->d.N, ctx->partial, ctx->dres, ctx->st, &ctx->prof);
     launch_scalar_scale(mismatch, 0.5 * ctx->h3(), ctx->dres, ctx->st, &ctx->prof);
     check_launch("mismatch_device");
+    ctx->reduction_in_flight();
     API_END(ctx)
 }
 
