@@ -134,8 +134,8 @@ int claire_mismatch_forward(claire_ctx *ctx, const float *v, float *m_final, dou
 /* Mismatch of the last claire_mismatch_forward without a synchronization:
  * writes 1/2 ||m(1) - m1||^2_{L2} to *mismatch, one double in DEVICE memory,
  * in order on the context's stream (the value claire_mismatch_forward returns
- * to the host).  CLAIRE_ERR_STATE before the first differentiable forward.  No
- * counterpart in the paper. */
+ * to the host).  CLAIRE_ERR_STATE before the first differentiable forward and
+ * once the images have been replaced after it.  No counterpart in the paper. */
 int claire_mismatch_device(claire_ctx *ctx, double *mismatch);
 
 /* Checkpoint stride the differentiable form of ctx uses (0 before its first
@@ -148,7 +148,8 @@ int claire_checkpoint_stride(const claire_ctx *ctx, int *stride);
  * of the state recomputed from its checkpoint, and the body force
  * int lambda grad m dt by the trapezoidal rule.  Writes the Euclidean gradient
  * grad_v = hx*hy*hz * int lambda grad m dt (float[3][N]) of
- * grad_mismatch * mismatch + <grad_m_final, m(1)>. */
+ * grad_mismatch * mismatch + <grad_m_final, m(1)>.  With a nonzero grad_mismatch,
+ * CLAIRE_ERR_STATE once the images have been replaced after that forward. */
 int claire_mismatch_backward(claire_ctx *ctx, double grad_mismatch, const float *grad_m_final,
                              float *grad_v);
 

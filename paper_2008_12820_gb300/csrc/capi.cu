@@ -957,6 +957,7 @@ struct claire_ctx {
     float *ck = nullptr, *seg_m = nullptr, *gbuf = nullptr, *bacc = nullptr, *lam2 = nullptr;
     int ck_stride = 0;
     bool ck_valid = false;
+    bool ck_images = false;  // m1 is still the one of the last differentiable forward
     int n_ck() const { return (nt + ck_stride - 1) / ck_stride + 1; }
     int ck_slot(int j) const { return j == nt ? n_ck() - 1 : j / ck_stride; }
     // floats of N the differentiable form holds for stride k
@@ -1032,11 +1033,16 @@ struct claire_ctx {
             src = dst;
             if (dst == a) { float *t = a; a = b; b = t; }
         }
-        ck_valid = true;
+        ck_valid = ck_images = true;
         const float *mT = ck + (size_t)ck_slot(nt) * N;
         if (m_final) CK(cudaMemcpyAsync(m_final, mT, N * sizeof(float), cudaMemcpyDeviceToDevice, st));
         check_launch("mismatch_forward");
         return want_mismatch ? mismatch_of(mT) : 0.0;
+    }
+
+    // the residual m1 - m(1) needs the image that the forward was compared with
+    void need_forward_images() const {
+        if (!ck_images) throw Error(CLAIRE_ERR_STATE, "the images changed after the last differentiable forward");
     }
 
     // backward of (mismatch, m(1)) -> v: adjoint from l(1) = gmis (m1 - m(1))
@@ -1046,6 +1052,8 @@ struct claire_ctx {
     // grad_v = h^3 b (Euclidean)
     void diff_backward(double gmis, const float *gm_final, float *grad_v) {
         if (!ck_valid) throw Error(CLAIRE_ERR_STATE, "no differentiable forward at this point");
+        // the upstream gradient of m(1) alone needs no image
+        if (gmis != 0.0) need_forward_images();
         const size_t N = d.N;
         const double H3 = h3();
         const float dt = 1.f / nt;
@@ -1316,6 +1324,7 @@ int claire_set_images(claire_ctx *ctx, const float *m0, const float *m1) {
     ctx->have_images = true;
     ctx->have_lin = false;
     ctx->gm0_valid = false;
+    ctx->ck_images = false;
     API_END(ctx)
 }
 
@@ -1396,6 +1405,7 @@ int claire_mismatch_device(claire_ctx *ctx, double *mismatch) {
     API_BEGIN(ctx)
     need(mismatch, "mismatch");
     if (!ctx->ck_valid) throw Error(CLAIRE_ERR_STATE, "no differentiable forward at this point");
+    ctx->need_forward_images();
     launch_sqdiff(ctx->diff_final(), ctx->m1, ctx->d.N, ctx->partial, ctx->dres, ctx->st, &ctx->prof);
     launch_scalar_scale(mismatch, 0.5 * ctx->h3(), ctx->dres, ctx->st, &ctx->prof);
     check_launch("mismatch_device");
@@ -1882,6 +1892,7 @@ int claire_solve_host(claire_ctx *ctx, const float *m0, const float *m1, const f
     ctx->have_images = true;
     ctx->have_lin = false;
     ctx->gm0_valid = false;
+    ctx->ck_images = false;
     struct ImgWait {
         claire_ctx *c;
         ~ImgWait() { c->wait_images(); }

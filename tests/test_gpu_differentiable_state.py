@@ -1,5 +1,5 @@
 """State that the differentiable transport keeps between calls: reductions that
-a call leaves in flight on its stream."""
+a call leaves in flight on its stream, and the images of the last forward."""
 import pytest
 import torch
 
@@ -43,3 +43,27 @@ def test_new_stream_waits_for_a_reduction_in_flight(C, problem):
         # and the context reduces as before on its new stream
         torch.cuda.synchronize()
         assert float(out) == mis and reg.mismatch_forward(v)[1] == mis
+
+
+def test_replaced_images_end_the_mismatch_of_the_last_forward(C, problem):
+    """Checkpoints of one pair and the reference image of another belong to no
+    mismatch; the upstream gradient of m(1) alone needs neither image."""
+    out = torch.zeros((), dtype=torch.float64, device="cuda")
+    v = 0.7 * problem["v_true"]
+    with C.Registration(SHAPE, NT, 1e-2, 1.0) as reg:
+        reg.set_images(problem["m0"], problem["m1"])
+        _, mis = reg.mismatch_forward(v)
+        of_m1 = reg.mismatch_backward(0.0, problem["m0"])
+        both = reg.mismatch_backward(1.0, problem["m0"])
+        reg.set_images(problem["m1"], problem["m0"])
+        for call in (lambda: reg._c("claire_mismatch_device", out.data_ptr()),
+                     lambda: reg.mismatch_backward(1.0), lambda: reg.mismatch_backward(1.0, problem["m0"])):
+            with pytest.raises(C.ClaireError) as e:
+                call()
+            assert e.value.code == 4
+        assert torch.equal(reg.mismatch_backward(0.0, problem["m0"]), of_m1)
+        reg.set_images(problem["m0"], problem["m1"])
+        assert reg.mismatch_forward(v)[1] == mis
+        assert torch.equal(reg.mismatch_backward(1.0, problem["m0"]), both)
+        reg._c("claire_mismatch_device", out.data_ptr())
+        assert float(out) == mis
