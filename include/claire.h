@@ -88,8 +88,8 @@ int claire_create_ex(int nx, int ny, int nz, int nt, double beta, double gamma, 
 int claire_destroy(claire_ctx *ctx);
 
 /* Order all later work of ctx on `stream` (a cudaStream_t; NULL = legacy).  The
- * new stream waits for a reduction that claire_mismatch_device left in flight on
- * the stream before; ordering anything else behind that stream is the caller's. */
+ * new stream waits for a reduction that a claire_mismatch_*device call left in
+ * flight on the stream before; ordering anything else behind that stream is the caller's. */
 int claire_set_stream(claire_ctx *ctx, void *stream);
 
 /* Change beta and gamma (same rules as claire_create); drops nothing but the
@@ -119,7 +119,7 @@ int claire_forward(claire_ctx *ctx, const float *v, float *m_final, double *mism
 
 /* Differentiable forward (Eq. 2.1b): m(1) from m0 along the characteristics
  * of v, keeping the state only every checkpoint_stride time steps (and at
- * t = 1); *mismatch = 1/2 ||m(1) - m1||^2_{L2} (nullable; synchronizes if given).
+ * t = 1); *mismatch = 1/2 ||m(1) - m1||^2_{L2} (nullable).  Synchronizes.
  * m_final: float[N] (nullable).  checkpoint_stride in [1, nt], or 0: chosen
  * from the memory left on the device (and under claire_set_workspace_limit)
  * -- every state kept (stride 1: the backward recomputes nothing) when that
@@ -130,6 +130,12 @@ int claire_forward(claire_ctx *ctx, const float *v, float *m_final, double *mism
  * dominates; keep it when it fits, recompute otherwise). */
 int claire_mismatch_forward(claire_ctx *ctx, const float *v, float *m_final, double *mismatch,
                             int checkpoint_stride);
+
+/* claire_mismatch_forward without a synchronization: *mismatch (nullable) is one
+ * double in DEVICE memory, written in order on the context's stream.  No
+ * counterpart in the paper. */
+int claire_mismatch_forward_device(claire_ctx *ctx, const float *v, float *m_final, double *mismatch,
+                                   int checkpoint_stride);
 
 /* Mismatch of the last claire_mismatch_forward without a synchronization:
  * writes 1/2 ||m(1) - m1||^2_{L2} to *mismatch, one double in DEVICE memory,

@@ -39,6 +39,7 @@ EXPORTED = [
     "claire_precond_h0", "claire_solve_continuation", "claire_set_discretization", "claire_solve_batch",
     "claire_mismatch_forward", "claire_mismatch_backward", "claire_solve_host", "claire_set_workspace_limit",
     "claire_checkpoint_stride", "claire_check_count", "claire_mismatch_device",
+    "claire_mismatch_forward_device",
 ]
 
 
@@ -108,6 +109,7 @@ def load(path: str = LIB_PATH):
         "claire_mismatch_forward": [P, V, V, pd, I],
         "claire_mismatch_backward": [P, D, V, V],
         "claire_mismatch_device": [P, V],
+        "claire_mismatch_forward_device": [P, V, V, V, I],
         "claire_checkpoint_stride": [P, ctypes.POINTER(ctypes.c_int)],
         "claire_check_count": [ctypes.POINTER(ctypes.c_ulonglong), I],
         "claire_solve_continuation": [P, V, D, D, D, ctypes.POINTER(SolveOpts),
@@ -336,8 +338,8 @@ class Registration:
         stream; torch's current stream is ordered behind it."""
         m, mis = self._new(), torch.empty((), dtype=torch.float64, device="cuda")
         self._behind_current()
-        self._c("claire_mismatch_forward", self._vec(v, "v"), self._scal(m, "m_final"), None, int(checkpoint_stride))
-        self._c("claire_mismatch_device", ctypes.c_void_p(mis.data_ptr()))
+        self._c("claire_mismatch_forward_device", self._vec(v, "v"), self._scal(m, "m_final"),
+                ctypes.c_void_p(mis.data_ptr()), int(checkpoint_stride))
         self._current_behind()
         return m, mis
 

@@ -1008,12 +1008,15 @@ struct claire_ctx {
         }
     }
 
-    // forward transport keeping only checkpoints; X-, X+ and c at v kept for
-    // the backward; returns the mismatch 1/2 ||m(1) - m1||^2.  stride 0: the
-    // stride is chosen from the free memory (auto_stride) at the first call
     // m(1) of the last differentiable forward
     const float *diff_final() const { return ck + (size_t)ck_slot(nt) * d.N; }
-    double diff_forward(const float *v, float *m_final, int stride, bool want_mismatch = true) {
+
+    // forward transport keeping only checkpoints; X-, X+ and c at v kept for
+    // the backward.  stride 0: the stride is chosen from the free memory
+    // (auto_stride) at the first call
+    void diff_forward(const float *v, float *m_final, int stride) {
+        if (stride < 0 || stride > nt)
+            throw Error(CLAIRE_ERR_ARG, "checkpoint_stride must be in [0, nt] (0: chosen from the free memory)");
         if (!have_images) throw Error(CLAIRE_ERR_STATE, "images not set (claire_set_images)");
         if (stride == 0) stride = ck_stride ? ck_stride : auto_stride();
         ensure_ck(stride);
@@ -1034,10 +1037,16 @@ struct claire_ctx {
             if (dst == a) { float *t = a; a = b; b = t; }
         }
         ck_valid = ck_images = true;
-        const float *mT = ck + (size_t)ck_slot(nt) * N;
-        if (m_final) CK(cudaMemcpyAsync(m_final, mT, N * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        if (m_final) CK(cudaMemcpyAsync(m_final, diff_final(), N * sizeof(float), cudaMemcpyDeviceToDevice, st));
         check_launch("mismatch_forward");
-        return want_mismatch ? mismatch_of(mT) : 0.0;
+    }
+
+    // mismatch of the last differentiable forward into device memory
+    void diff_mismatch(double *mismatch) {
+        launch_sqdiff(diff_final(), m1, d.N, partial, dres, st, &prof);
+        launch_scalar_scale(mismatch, 0.5 * h3(), dres, st, &prof);
+        check_launch("mismatch_device");
+        reduction_in_flight();
     }
 
     // the residual m1 - m(1) needs the image that the forward was compared with
@@ -1394,10 +1403,18 @@ int claire_mismatch_forward(claire_ctx *ctx, const float *v, float *m_final, dou
                             int checkpoint_stride) {
     API_BEGIN(ctx)
     need(v, "v");
-    if (checkpoint_stride < 0 || checkpoint_stride > ctx->nt)
-        throw Error(CLAIRE_ERR_ARG, "checkpoint_stride must be in [0, nt] (0: chosen from the free memory)");
-    const double mis = ctx->diff_forward(v, m_final, checkpoint_stride, mismatch != nullptr);
-    if (mismatch) *mismatch = mis;
+    ctx->diff_forward(v, m_final, checkpoint_stride);
+    if (mismatch) *mismatch = ctx->mismatch_of(ctx->diff_final());
+    else CK(cudaStreamSynchronize(ctx->st));
+    API_END(ctx)
+}
+
+int claire_mismatch_forward_device(claire_ctx *ctx, const float *v, float *m_final, double *mismatch,
+                                   int checkpoint_stride) {
+    API_BEGIN(ctx)
+    need(v, "v");
+    ctx->diff_forward(v, m_final, checkpoint_stride);
+    if (mismatch) ctx->diff_mismatch(mismatch);
     API_END(ctx)
 }
 
@@ -1406,10 +1423,7 @@ int claire_mismatch_device(claire_ctx *ctx, double *mismatch) {
     need(mismatch, "mismatch");
     if (!ctx->ck_valid) throw Error(CLAIRE_ERR_STATE, "no differentiable forward at this point");
     ctx->need_forward_images();
-    launch_sqdiff(ctx->diff_final(), ctx->m1, ctx->d.N, ctx->partial, ctx->dres, ctx->st, &ctx->prof);
-    launch_scalar_scale(mismatch, 0.5 * ctx->h3(), ctx->dres, ctx->st, &ctx->prof);
-    check_launch("mismatch_device");
-    ctx->reduction_in_flight();
+    ctx->diff_mismatch(mismatch);
     API_END(ctx)
 }
 

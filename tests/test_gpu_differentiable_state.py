@@ -1,5 +1,6 @@
 """State that the differentiable transport keeps between calls: reductions that
-a call leaves in flight on its stream, and the images of the last forward."""
+a call leaves in flight on its stream, and the images of the last forward; and
+which of its calls return behind their work."""
 import pytest
 import torch
 
@@ -66,4 +67,28 @@ def test_replaced_images_end_the_mismatch_of_the_last_forward(C, problem):
         assert reg.mismatch_forward(v)[1] == mis
         assert torch.equal(reg.mismatch_backward(1.0, problem["m0"]), both)
         reg._c("claire_mismatch_device", out.data_ptr())
+        assert float(out) == mis
+
+
+def test_mismatch_forward_returns_behind_its_work(C, problem):
+    """claire_mismatch_forward synchronizes whether or not the mismatch is asked
+    for; claire_mismatch_forward_device does not."""
+    a = torch.cuda.Stream()
+    v = 0.7 * problem["v_true"]
+    m, out = torch.empty(SHAPE, device="cuda"), torch.zeros((), dtype=torch.float64, device="cuda")
+    with C.Registration(SHAPE, NT, 1e-2, 1.0, stream=a) as reg:
+        torch.cuda.synchronize()
+        reg.set_images(problem["m0"], problem["m1"])
+        ref, mis = reg.mismatch_forward(v)
+        args = reg._vec(v), reg._scal(m)
+        for name, mismatch, behind in (("claire_mismatch_forward", None, True),
+                                       ("claire_mismatch_forward_device", out.data_ptr(), False)):
+            m.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(a):
+                torch.cuda._sleep(DELAY)
+            reg._c(name, *args, mismatch, 2)
+            assert a.query() is behind
+            torch.cuda.synchronize()
+            assert torch.equal(m, ref)
         assert float(out) == mis
