@@ -1285,7 +1285,7 @@ int claire_create_ex(int nx, int ny, int nz, int nt, double beta, double gamma, 
         c->partial = (double *)c->alloc_bytes(kPartialDoubles * sizeof(double));
         CK(cudaMemset(c->partial, 0, kPartialDoubles * sizeof(double)));
         CK(cudaStreamSynchronize(0));  // before work on any other stream can use it
-        c->dres = (double *)c->alloc_bytes(16 * sizeof(double));
+        c->dres = c->partial + 4 * kReduceBlocks;  // slots 0 to 12 in use
         c->dflag = (int *)c->alloc_bytes(sizeof(int));
         c->ntiles = tile_count(c->d);
         c->rng = (int4 *)c->alloc_bytes((size_t)4 * c->ntiles * sizeof(int4));

@@ -263,7 +263,10 @@ void launch_pcg_dir_u0(float *p, float *Ap, const float *z, const float *r, cons
 void launch_h0_apply(float *q, const float *Ap, const float *gm, const float *p, long long N, double *partial,
                      double *dev_out, cudaStream_t st, Profiler *prof);
 constexpr int kReduceBlocks = 1216;  // 152 SMs x 8
-constexpr int kPartialDoubles = 4 * kReduceBlocks + 1;  // block partials and the ticket of the last block
+// The reduction buffer of a context: block partials, 16 results, of which the
+// last one's place holds the ticket of the last block
+constexpr int kPartialDoubles = 4 * kReduceBlocks + 16;
+constexpr int kTicket = kPartialDoubles - 1;
 
 // grid of a persistent transform pass: as many blocks as fit the SMs at this
 // shared memory per block (227 KB per SM, 1 KB reserved per block, at most 8

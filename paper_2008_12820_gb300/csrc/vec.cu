@@ -487,9 +487,9 @@ __global__ void k_h2f(const __half *__restrict__ in, float *__restrict__ out, lo
         out[i] = __half2float(in[i]);
 }
 
-// the ticket of last_block, behind the partial sums (zeroed with the context;
-// launches that share a partial buffer run in order on one stream)
-inline unsigned *ticket_of(double *partial) { return reinterpret_cast<unsigned *>(partial + 4 * kReduceBlocks); }
+// the ticket of last_block, behind the partial sums and results (zeroed with the
+// context; launches that share a partial buffer run in order on one stream)
+inline unsigned *ticket_of(double *partial) { return reinterpret_cast<unsigned *>(partial + kTicket); }
 
 inline int blocks_for(long long n) {
     long long b = (n + RT - 1) / RT;
