@@ -280,7 +280,7 @@ __device__ __forceinline__ float gather_lean(const T *__restrict__ f, const Dims
 // the pending loads hold up the shared loads behind them).  The 64 taps of a
 // voxel are shared-memory reads with immediate offsets, the same instruction
 // stream for every lane (the periodic wrap happened once, when the box was
-// fetched).  A thread sums two voxels at a time on the paired FP32
+// fetched).  A thread sums two voxels at a time (SlPair) on the paired FP32
 // instructions, weights included (212 warp instructions per 32 voxels instead
 // of 266).  What bounds the state step is the shared-memory pipe: 64 tap
 // wavefronts per 32 voxels, 10 more of bank conflicts where floors change
@@ -621,6 +621,16 @@ template <int MODE> struct SlShare {
     static constexpr bool v = MODE == SL_PLAIN || MODE == SL_ADJFAC;
 };
 
+// Steps that sum a thread's voxels in pairs: all but the incremental state's,
+// which hold six inputs a voxel at three blocks per SM and lose more to the
+// pair's registers than its instructions save.  One voxel after the other
+// there (the same operations): incremental state of a matvec 905 -> 880 us at
+// 256^3 (its last step 270 -> 246), 572 -> 558 at 200x180x162, 531 -> 501 at
+// 160^3 with FP16 trajectories and eight steps.
+template <int MODE> struct SlPair {
+    static constexpr bool v = MODE != SL_INCSTATE && MODE != SL_INCLAST;
+};
+
 // floors inside the clamp of floor_int: a non-finite or huge displacement
 // (clamped to +-1e6 there, while the box path converts floorf directly) sends
 // the tile to the gather path, whose stencil clamps
@@ -829,6 +839,16 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
                     } else if (ORDER == 1) {
                         acc.x = box_linear(smem + o[0], u[0].x, u[1].x, u[2].x);
                         acc.y = box_linear(smem + o[1], u[0].y, u[1].y, u[2].y);
+                    } else if (!SlPair<MODE>::v) {
+                        float w1[4], w2[4], w3[4];
+                        lagrange4(u[0].x, w1);
+                        lagrange4(u[1].x, w2);
+                        lagrange4(u[2].x, w3);
+                        acc.x = box_cubic<BOX_PITCH>(smem + o[0], w1, w2, w3);
+                        lagrange4(u[0].y, w1);
+                        lagrange4(u[1].y, w2);
+                        lagrange4(u[2].y, w3);
+                        acc.y = box_cubic<BOX_PITCH>(smem + o[1], w1, w2, w3);
                     } else {
                         float2 w1[4], w2[4], w3[4];
                         lagrange4x2(u[0], w1);
