@@ -268,7 +268,7 @@ __device__ __forceinline__ float gather_lean(const T *__restrict__ f, const Dims
 
 // ---------------------------------------------------------------------------
 // Software-pipelined tiled semi-Lagrangian step (the production path).
-// Blocks walk consecutive tiles of 32 x 8 x 4 voxels (sl_chunk).  Every tile
+// Blocks walk consecutive tiles of 32 x 8 x 4 voxels (sl_grid).  Every tile
 // has a box entry (written by the foot-point kernel with the displacements, or
 // by k_tile_ranges): the smallest floor of its displacements per axis, which
 // fixes where its shared-memory source box starts, and whether the floors
@@ -715,7 +715,7 @@ constexpr int GTAB = 64;  // box entries a block stages in shared memory at a ti
 // tile needs a bounds check (measured ~5% of the step time at 256^3)
 template <int MODE, int ORDER, typename TS = float, typename TG = float, bool FULL = false>
 __global__ void __launch_bounds__(PT3 * PT2, SlOcc<MODE>::v)
-k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked_in, int chunk) {
+k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked_in, int chunk, int extra) {
     static_assert(std::is_same<TS, float>::value, "the box path stages FP32 source fields");
     constexpr int NE = EpiCount<MODE>::v > 0 ? EpiCount<MODE>::v : 1;
     constexpr int NX = EarlyCount<MODE>::v > 0 ? EarlyCount<MODE>::v : 1;
@@ -726,7 +726,8 @@ k_sl_pipe(SlArgsT<TS, TG> a, Dims d, const int4 *__restrict__ tiles, int chunked
     const int nb3 = (d.n3 + PT3 - 1) / PT3, nb2 = (d.n2 + PT2 - 1) / PT2, nb1 = (d.n1 + PT1 - 1) / PT1;
     const int ntiles = nb3 * nb2 * nb1;
     const long long N = d.N, plane = (long long)d.n2 * d.n3;
-    const int tbeg = min(ntiles, (int)blockIdx.x * chunk), tend = min(ntiles, tbeg + chunk);
+    const int tbeg = (int)blockIdx.x * chunk + min((int)blockIdx.x, extra);
+    const int tend = min(ntiles, tbeg + chunk + ((int)blockIdx.x < extra ? 1 : 0));
     if (tbeg < tend) {
         // box of a tile at its own floor range g (lo1, lo2, lo3); a tile whose
         // range does not fit (g.w == 0) copies nothing
@@ -1157,13 +1158,25 @@ inline int chunk_ok(const Dims &d, const T *f) {
 // 88); the accumulating adjoint steps (two blocks per SM) 240 -> 234 at 256^3
 // with 8 (4: 236), and no gain at 192^3 (109 both).  A new block exposes its
 // first loads, so with fewer tiles to a slot (128^3: 4.5; state 33.7 with equal
-// shares, 35.5 with 4 tiles) every block takes an equal share of one wave.
+// shares, 35.5 with 4 tiles) every block takes an equal share of one wave: as
+// equal as whole tiles allow from three tiles on (rounded up to the same for
+// all, the last SMs get a block less: the four state steps of a forward take
+// 143 against 131 us at 128^3, 215 against 188 at 144^3, 221 against 220 at
+// 160^3), rounded up below, where a block of two tiles that overlap beats two
+// blocks of one (80^3: 67 us, 81 with one or two tiles a block).
 // At most 4 kReduceBlocks blocks: a dot-product step leaves one partial sum each.
-inline int sl_chunk(long long ntiles, int slots, bool two_per_sm) {
+// Block b takes chunk tiles, and one more if b < extra.
+struct SlGrid {
+    int blocks, chunk, extra;
+};
+inline SlGrid sl_grid(long long ntiles, int slots, bool two_per_sm) {
     const int few = two_per_sm ? 8 : 4;
     const long long share = (ntiles + slots - 1) / slots;
-    const long long chunk = share > (two_per_sm ? 32 : 12) ? few : share;
-    return (int)std::max<long long>(chunk, (ntiles + 4 * kReduceBlocks - 1) / (4 * kReduceBlocks));
+    if (share <= (two_per_sm ? 32 : 12) && share >= 3)
+        return SlGrid{slots, (int)(ntiles / slots), (int)(ntiles % slots)};
+    const long long least = (ntiles + 4 * kReduceBlocks - 1) / (4 * kReduceBlocks);
+    const long long chunk = share < 3 ? share : std::max<long long>(few, least);
+    return SlGrid{(int)((ntiles + chunk - 1) / chunk), (int)chunk, 0};
 }
 
 // returns the number of blocks launched (the partial sums a dot-product step
@@ -1174,10 +1187,10 @@ int launch_pipe_f(const Dims &d, const SlArgsT<TS, TG> &a, const int4 *tiles, cu
     // the shared-memory limit is set once per instantiation and device
     static SmemAttr attr;
     attr.ensure(k_sl_pipe<MODE, ORDER, TS, TG, FULL>, (int)smem, "k_sl_pipe");
-    const int chunk = sl_chunk(tile_count(d), SlOcc<MODE>::v * num_sms(), SlOcc<MODE>::v == 2);
-    const int grid = (int)((tile_count(d) + chunk - 1) / chunk);
-    k_sl_pipe<MODE, ORDER, TS, TG, FULL><<<grid, dim3(PT3, PT2), smem, st>>>(a, d, tiles, chunk_ok(d, a.src), chunk);
-    return grid;
+    const SlGrid g = sl_grid(tile_count(d), SlOcc<MODE>::v * num_sms(), SlOcc<MODE>::v == 2);
+    k_sl_pipe<MODE, ORDER, TS, TG, FULL><<<g.blocks, dim3(PT3, PT2), smem, st>>>(a, d, tiles, chunk_ok(d, a.src),
+                                                                                g.chunk, g.extra);
+    return g.blocks;
 }
 
 // kernels one SL step launches
