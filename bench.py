@@ -59,18 +59,25 @@ ERR_CHECK_N = 128        # GPU vs oracle gradient / matvec on a 128^3 instance
 KCLASS = ["footpoint", "state", "adjoint", "incstate", "incadj", "bodyforce", "fft_r2c",
           "fft_c2c", "fft_mul", "fft_c2r", "reduce", "vector", "interp", "fd", "deriv"]
 # kernel function names of each class (for the ncu summaries); the template
-# argument of k_sl_pipe is the step kind: 0 plain, 1 adjoint, 2 incremental
-# state, 3 adjoint factor, 4 last incremental-state step, 5 adjoint step that
-# adds its body-force term, 6 the same with the curvature dot
+# argument of k_sl_pipe is the step kind: 0 plain, 2 incremental state, 3 adjoint
+# factor, 4 last incremental-state step, 5 adjoint step that adds its body-force
+# term, 6 the same with the curvature dot.  Transforms: kr_* lengths 16 G, kg_* other
+# lengths with a two-step plan, k_* the staged form of the rest
 KNAMES = {"footpoint": "k_footpoints_box, k_footpoints, k_tile_ranges, k_sl_pipe<3, *>",
-          "state": "k_sl_pipe<0, *>", "adjoint": "k_sl_pipe<5, *>", "incstate": "k_sl_pipe<2, *>, k_sl_pipe<4, *>",
-          "incadj": "k_sl_pipe<5, *>, k_sl_pipe<6, *>", "bodyforce": "k_adjfinal_acc",
-          "fft_r2c": "k_r2c_x3_p (k_r2c_x3 for unaligned rows)", "fft_c2c": "k_c2c_x2", "fft_mul": "k_mul_x1",
-          "fft_c2r": "k_c2r_x3_p (k_c2r_x3 for unaligned spectra)",
-          "reduce": "k_reduce2, k_stats, k_finalize, k_finalize4",
-          "vector": "k_pcg_update, k_pcg_dir_u0, k_axpby, k_incstate_init, k_f2h, k_h2f",
+          "state": "k_sl_pipe<0, *>", "adjoint": "k_sl_pipe<5, *>, k_sl_pipe<6, *>",
+          "incstate": "k_sl_pipe<2, *>, k_sl_pipe<4, *>",
+          "incadj": "k_sl_pipe<5, *>, k_sl_pipe<6, *>, k_finalize", "bodyforce": "k_adjfinal_acc, k_bodyforce_start",
+          "fft_r2c": "kr_r2c (kr_plane_fwd, kg_r2c, k_r2c_x3_p, k_r2c_x3)",
+          "fft_c2c": "kr_c2c (kg_c2c, k_c2c_x2, k_c2c_x2_ip)",
+          "fft_mul": "kr_mul (kg_mul, k_mul_x1, k_mul_x1_ip, k_spec_restrict, k_spec_twolevel)",
+          "fft_c2r": "kr_c2r (kr_plane_inv, kg_c2r, k_c2r_x3_p, k_c2r_x3)",
+          "reduce": "k_reduce2, k_stats, k_ls_dots, k_inner_init, k_inner_ctl, k_pcg_ctl, k_pcg_ctl_init, "
+                    "k_scalar_copy, k_scalar_set",
+          "vector": "k_pcg_update, k_pcg_dir_u0, k_pcg_dir, k_pcg_negcopy, k_h0_apply, k_axpby, k_diff_flag, "
+                    "k_incstate_init, k_adjoint_final, k_scalar_scale, k_f2h, k_h2f",
           "interp": "k_sl_pipe<0, *>", "fd": "k_grad_fd8, k_div_fd8",
-          "deriv": "k_deriv_x3_p, k_deriv_strided_p (k_deriv_x3, k_deriv_strided for unaligned rows)"}
+          "deriv": "kr_deriv_x3, kr_deriv_strided (kg_deriv_x3, kg_deriv_strided, k_deriv_x3, k_deriv_x3_p, "
+                   "k_deriv_strided, k_deriv_strided_p, k_deriv_strided_ip)"}
 
 
 # the transport and transform classes (every one of them is asked to reach
