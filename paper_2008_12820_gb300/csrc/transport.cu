@@ -156,7 +156,6 @@ __device__ __forceinline__ int floor_int(float x) {
 
 // One thread per voxel (the trilinear form); the box geometry of its outputs
 // comes from k_tile_ranges.
-template <int ORDER>
 __global__ void __launch_bounds__(BX * BY)
 k_footpoints(const float *__restrict__ v, float *__restrict__ dispm, float *__restrict__ dispp,
              Dims d, float dt, float ih1, float ih2, float ih3) {
@@ -171,20 +170,9 @@ k_footpoints(const float *__restrict__ v, float *__restrict__ dispm, float *__re
         if (!out) continue;
         const float sg = s == 0 ? -1.f : 1.f;
         const float q1 = sg * dt * v1 * ih1, q2 = sg * dt * v2 * ih2, q3 = sg * dt * v3 * ih3;
-        float w1, w2, w3;
-        if (ORDER == 1) {
-            w1 = gather8(v, d, p.i1, p.i2, p.i3, q1, q2, q3);
-            w2 = gather8(v + N, d, p.i1, p.i2, p.i3, q1, q2, q3);
-            w3 = gather8(v + 2 * N, d, p.i1, p.i2, p.i3, q1, q2, q3);
-        } else {
-            Axis4 a1, a2, a3;
-            axis_stencil(p.i1, q1, d.n1, d.n2 * d.n3, a1);
-            axis_stencil(p.i2, q2, d.n2, d.n3, a2);
-            axis_stencil(p.i3, q3, d.n3, 1, a3);
-            w1 = gather64(v, a1, a2, a3);
-            w2 = gather64(v + N, a1, a2, a3);
-            w3 = gather64(v + 2 * N, a1, a2, a3);
-        }
+        const float w1 = gather8(v, d, p.i1, p.i2, p.i3, q1, q2, q3);
+        const float w2 = gather8(v + N, d, p.i1, p.i2, p.i3, q1, q2, q3);
+        const float w3 = gather8(v + 2 * N, d, p.i1, p.i2, p.i3, q1, q2, q3);
         const float hs = 0.5f * sg * dt;
         out[p.id] = hs * (v1 + w1) * ih1;
         out[N + p.id] = hs * (v2 + w2) * ih2;
@@ -632,8 +620,8 @@ template <int MODE> struct SlPair {
 };
 
 // floors inside the clamp of floor_int: a non-finite or huge displacement
-// (clamped to +-1e6 there, while the box path converts floorf directly) sends
-// the tile to the gather path, whose stencil clamps
+// (clamped to +-1e6 there) sends the tile to the gather path, whose stencil
+// clamps; the box path takes the floor by FLOOR_MAGIC, which needs less than 2^22
 __device__ __forceinline__ bool floor_sane(int lo, int hi) { return lo > -1000000 && hi < 1000000; }
 
 // Box entry of one tile of a displacement field: {lo1, lo2, lo3, ok}, lo_d =
@@ -1203,9 +1191,7 @@ inline bool full_tiles(const Dims &d) { return d.n3 % PT3 == 0 && d.n2 % PT2 == 
 // incremental state 13.8 -> 10.4 ms per 256^3 solve)
 template <int MODE, int ORDER, typename TS, typename TG>
 int launch_pipe_o(const Dims &d, const SlArgsT<TS, TG> &a, const int4 *tiles, cudaStream_t st) {
-    if constexpr (ORDER == 3 || ORDER == 1) {
-        if (full_tiles(d)) return launch_pipe_f<MODE, ORDER, TS, TG, true>(d, a, tiles, st);
-    }
+    if (full_tiles(d)) return launch_pipe_f<MODE, ORDER, TS, TG, true>(d, a, tiles, st);
     return launch_pipe_f<MODE, ORDER, TS, TG, false>(d, a, tiles, st);
 }
 
@@ -1293,7 +1279,7 @@ void launch_footpoints(const Dims &d, int nt, const float *v, float *dispm, floa
         {
             ProfScope ps(prof, CLAIRE_K_FOOTPOINT, st, (double)d.N * (12 + (dispm ? 12 : 0) + (dispp ? 12 : 0)), 1);
             const dim3 grid((d.n3 + BX - 1) / BX, (d.n2 + BY - 1) / BY, d.n1);
-            k_footpoints<1><<<grid, dim3(BX, BY), 0, st>>>(v, dispm, dispp, d, dt, i1, i2, i3);
+            k_footpoints<<<grid, dim3(BX, BY), 0, st>>>(v, dispm, dispp, d, dt, i1, i2, i3);
         }
         if (dispm) launch_tile_ranges(d, dispm, tiles_m, st, prof);
         if (dispp) launch_tile_ranges(d, dispp, tiles_p, st, prof);
