@@ -13,9 +13,9 @@
 //   4. x2 inverse, in place.
 //   5. x3 inverse, half spectrum -> real, two lines per complex transform,
 //      with an optional addend in the epilogue.
-// Lengths 32, 64, 96, 128, 160, 192 and 256 (fft_reg.cuh) and the other products
-// of 2, 3 and 5 from 36 to 240 (fft_gen.cuh) run in registers around one exchange
-// through shared memory.  At the other lengths a pass stages a tile of whole
+// Lengths 32, 64, 96, 128, 160, 192 and 256 (fft_reg.cuh) and 22 others from 36 to
+// 240 (listed in fft_gen.cuh) run in registers around one exchange
+// through shared memory.  At the remaining lengths a pass stages a tile of whole
 // lines in shared memory and runs a mixed-radix Stockham FFT there.  Either way:
 // natural-order output, no bit reversal, twiddles from a table computed in
 // double on the host.
@@ -514,7 +514,8 @@ k_c2r_x3_p(const float2 *__restrict__ in, TO *__restrict__ out, const float *__r
 // forms they replace at these lengths were bound by shared-memory round trips,
 // barriers and issue.  Per pass over three components, before and after:
 //   256^3 (59 us at the copy rate)  x3 forward 90 -> 66 us, x2 81 -> 70,
-//         x1 with multiplier 145 -> 121, x3 inverse 117 -> 78 (with addend)
+//         x1 with multiplier 145 -> 121, x3 inverse 117 -> 78 (mean of
+//         calls without and with an addend, which is another 30 us of bytes)
 //   192^3 (25 us)  50 -> 36, 61 -> 32, 93 -> 54, 64 -> 40
 //   128^3 (7.5 us, and about 5 us of launch)  19 -> 15, 16.5 -> 12, 26 -> 19, 21 -> 13
 // The x3 and x2 passes are within 0.75-0.9 of the copy rate at 256^3; the x1

@@ -1,5 +1,8 @@
-// fft_gen.cuh -- two-step register transforms for the lengths 36 ... 240 that
-// are products of 2, 3 and 5 but not 16 G (fft_reg.cuh).
+// fft_gen.cuh -- two-step register transforms for 22 lengths that are not 16 G
+// (fft_reg.cuh): 36, 40, 45, 48, 50, 54, 60, 72, 75, 80, 90, 100, 108, 120, 135,
+// 144, 150, 180, 200, 216, 225 and 240.  The list (fft_gen*.cu) ends there because
+// these were instantiated and measured; 81, 125, 162, 243, 250, the lengths below
+// 32 and those above 256 take the staged plans.
 //
 // The radices of the runtime plan (4s, then 2, 3s, 5s) are split into two
 // groups with products G1 and G2, as equal as their order allows: step 1 takes
@@ -7,7 +10,7 @@
 // G1 j + r), step 2, after one exchange through shared memory, the second group
 // on k + G1 m (outputs k + G1 m in natural order).  Butterflies, twiddles and
 // order of operations are those of the staged runtime plan, which these passes
-// replace at these lengths (bit for bit the same); its stages of radix at most
+// replace at these lengths; its stages of radix at most
 // 5 took a shared-memory round trip, a barrier and run-time index divisions
 // each.  Three components, before and after: 240^3 x3 forward 181 -> 91 us, x2
 // 161 -> 67, x1 with multiplier 358 -> 127, x3 inverse 239 -> 109, derivatives

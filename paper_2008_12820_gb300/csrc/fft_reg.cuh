@@ -13,8 +13,11 @@
 // k = j, j + G, ... are the elements j + G r that step 1 of the inverse
 // transform needs: forward step 2, a pointwise multiplier and inverse step 1
 // then run back to back in registers.  Butterflies, twiddles and the order of
-// operations are those of the staged plans (radix_at), so the results are bit
-// for bit the same.
+// operations are those of the staged plans (radix_at).  When these passes came in,
+// gradients, divergences, beta A and its inverse, matvecs and transported images
+// were compared with the staged plans' and equal bit for bit on every grid tried;
+// the x1 transforms without a multiplier (two-level preconditioner) may fuse other
+// products: results 3e-8 to 1e-6 apart, both 4e-7 from 64 bits.
 //
 // Shared-memory layout: element e of a line lies at row e + e / 16.  With the
 // lines innermost (strided passes) row stride TL, with the elements innermost

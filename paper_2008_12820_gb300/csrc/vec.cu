@@ -8,7 +8,8 @@
 // once, a block reduces in FP64 by warp shuffles, block partials go to a
 // fixed-size array, and the block that finishes last sums them in a fixed
 // order: deterministic for a given grid.  (A second kernel for that sum cost
-// 3-4 us a reduction, a tenth of an inner PCG iteration on a 64^3 grid.)
+// 3-4 us a reduction, a tenth of an inner PCG iteration on a 64^3 grid; the
+// adjoint step with a dot product, transport.cu, still has one, k_finalize.)
 #include <cuda_fp16.h>
 #include <cstdint>
 #include <cuda_runtime.h>
