@@ -35,6 +35,7 @@ class TransportMismatch(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad_mis, grad_m1):
         reg = ctx.reg
+        # one host read: claire_mismatch_backward takes (and checks) a host scalar
         gmis = float(grad_mis) if grad_mis is not None else 0.0
         gm = None if grad_m1 is None else grad_m1.contiguous().float()
         reg._behind_current()

@@ -518,7 +518,7 @@ k_c2r_x3_p(const float2 *__restrict__ in, TO *__restrict__ out, const float *__r
 //         calls without and with an addend, which is another 30 us of bytes)
 //   192^3 (25 us)  50 -> 36, 61 -> 32, 93 -> 54, 64 -> 40
 //   128^3 (7.5 us, and about 5 us of launch)  19 -> 15, 16.5 -> 12, 26 -> 19, 21 -> 13
-// The x3 and x2 passes are within 0.75-0.9 of the copy rate at 256^3; the x1
+// The x3 and x2 passes are within 0.84-0.88 of the copy rate at 256^3 inside a solve; the x1
 // pass is bound by its registers (96 data values a thread, 12 warps per SM).
 
 // x2 transform (S = 0: direction s) and the x1 transform without a multiplier
